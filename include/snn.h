@@ -99,14 +99,21 @@ typedef struct snn_stats {
   uint64_t kernel_launches;/* kernels launched on this network's behalf (graph nodes included) */
 } snn_stats;
 
-/* Launch shapes; chosen by snn_autotune or set explicitly. */
+/* Launch shapes; chosen by snn_autotune or set explicitly.  A network starts on
+ * path 0 with the shape fields (update_block, deliver_warps, deliver_lanes,
+ * update_groups, deliver_blocks, overlap) at their defaults, which leaves the
+ * form to the library: networks whose neuron state fits the GPU's shared memory
+ * (about 2 million neurons in all) advance a window of steps in one launch of
+ * the persistent kernel, larger ones take two kernels per step.  Any other
+ * values of those fields run two kernels per step in that shape. */
 typedef struct snn_launch {
-  int32_t path;            /* 0 = two kernels per step (update, deliver); 1 = fused step kernel */
+  int32_t path;            /* 0 = two kernels per step (update, deliver), or the persistent kernel where the shape
+                              fields are at their defaults; 1 = persistent kernel where it fits */
   int32_t update_block;    /* threads per update block: 64 (update_groups 1 only), 128, 256 or 512 */
   int32_t deliver_warps;   /* warps per delivery block: 1..16 */
-  int32_t fused_block;     /* threads per fused-step block: 128..512 */
-  int32_t fused_items_per_sm; /* fused blocks per SM to launch (1..32, capped by occupancy) */
-  int32_t window_steps;    /* steps per captured CUDA graph (1..4096) */
+  int32_t fused_block;     /* path 1: threads per SM = fused_block * fused_items_per_sm, at most 1024; */
+  int32_t fused_items_per_sm; /* fused_block 128..512, fused_items_per_sm 1..32 */
+  int32_t window_steps;    /* steps per window: one launch or captured CUDA graph (1..4096) */
   int32_t deliver_lanes;   /* lanes that share one (spike, delay) segment of records: 4, 8, 16, 32 */
   int32_t update_groups;   /* groups of 4 neurons per update thread: 1, 2 or 4
                               (512-thread blocks: 1 or 2) */
@@ -135,8 +142,8 @@ int snn_set_allocator(snn_alloc_fn alloc, snn_free_fn free_fn, void *ctx);
 
 /* Device bytes a network with these parameters will hold once built
  * (synapse records and their delay-group table, neuron state, 2 max(1, min_delay)
- * input buffers, spike history of the last n_delay + max(1, min_delay) steps,
- * tables, recording buffers). */
+ * input buffers and 4 more for the persistent kernel, spike history of the last
+ * n_delay + max(1, min_delay) steps, tables, recording buffers). */
 int snn_footprint(const snn_params *p, size_t *bytes_out);
 
 /* Build a network on the device (Sec. 2.1 initialisation; Eq. 1 connectivity,
@@ -159,17 +166,20 @@ int snn_build_network(const snn_params *p, uint64_t seed, void *cuda_stream, snn
  * refractory period of at least one step), SNN_ERR_CUDA. */
 int snn_run(snn_handle h, uint64_t steps);
 
-/* Advance n networks together by steps[i] each with one fused kernel per time
- * step over all of them (networks that reach their count stop early).  Each
- * network's results are identical to snn_run on it alone.  The networks must
- * share one device; the call is ordered on the first network's stream.
+/* Advance n networks together by steps[i] each, in lockstep in one launch of
+ * the persistent kernel per window (networks that reach their count stop
+ * early; networks of different smallest delays, or more than fit one launch,
+ * take turns).  Each network's results are identical to snn_run on it alone.
+ * The networks must share one device; the call is ordered on the first
+ * network's stream.
  * Errors as snn_run, plus SNN_ERR_ARG (a network twice or NULL) and
  * SNN_ERR_LIMIT (more than 65535 networks).  The paper has no counterpart:
  * batching independent networks is a systems pattern of this library. */
 int snn_run_batch(const snn_handle *hs, const uint64_t *steps, int32_t n);
 
-/* Advance n networks by steps[i] each on the two-kernel path (launch path 0
- * for all of them, else SNN_ERR_ARG), every network on its own stream: the
+/* Advance n networks by steps[i] each on launch path 0 (for all of them, else
+ * SNN_ERR_ARG).  Networks that all have the default shape advance as in
+ * snn_run_batch.  Otherwise every network runs on its own stream: the
  * windows of the networks are issued round robin, so kernels of different
  * networks run at the same time when their streams differ (networks sharing a
  * stream run one after the other).  Each network's results
@@ -219,7 +229,7 @@ int snn_set_launch(snn_handle h, const snn_launch *cfg);
 /* Time candidate launch shapes on this network for `trial_steps` steps each
  * and keep the fastest; the network's state, counters and records are
  * restored afterwards, so results are unchanged.  Stages: update shapes (and
- * fused-path shapes), then delivery shapes for the best update shape, each
+ * path 1 shapes), then delivery shapes for the best update shape, each
  * stage timing every candidate once and its four fastest again (best of
  * three); then the L2 window and the kernel overlap switched off only when
  * that is at least 3% faster.  The result replaces the current shape only if
@@ -227,12 +237,12 @@ int snn_set_launch(snn_handle h, const snn_launch *cfg);
 int snn_autotune(snn_handle h, uint32_t trial_steps);
 
 /* The same with the launch path fixed: path 0 tunes the two-kernel path only
- * (the shapes snn_run_concurrent can run), 1 the fused path only, -1 both
+ * (the shapes snn_run_concurrent can run), 1 path 1 only, -1 both
  * (= snn_autotune).  The paper has no counterpart of the tuners. */
 int snn_autotune_path(snn_handle h, uint32_t trial_steps, int32_t path);
 
-/* The same for a batch advanced by snn_run_batch: fused-kernel shapes (block
- * size, blocks per SM, delivery chunk) are timed on the whole batch for
+/* The same for a batch advanced by snn_run_batch: path 1 shapes (threads per
+ * SM) are timed on the whole batch for
  * `trial_steps` steps each, from snapshots of every network (state, counters
  * and records restored afterwards, so results are unchanged); the fastest
  * shape replaces the first network's current shape only if at least 3%

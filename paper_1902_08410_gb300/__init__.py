@@ -229,8 +229,7 @@ class Network:
 
 
 def run_concurrent(nets, steps) -> None:
-    """Advance several networks on the two-kernel path, each on its own stream,
-    with their kernels overlapping on the GPU (see snn_run_concurrent)."""
+    """Advance several networks on launch path 0 side by side (see snn_run_concurrent)."""
     nets = list(nets)
     if isinstance(steps, int):
         steps = [steps] * len(nets)
@@ -240,7 +239,7 @@ def run_concurrent(nets, steps) -> None:
 
 
 def autotune_batch(nets, trial_steps: int = 200) -> dict:
-    """Choose the fused-kernel shape for a batch (see snn_autotune_batch); returns it."""
+    """Choose the path 1 shape for a batch (see snn_autotune_batch); returns it."""
     nets = list(nets)
     hs = (ctypes.c_void_p * len(nets))(*[n.handle.value for n in nets])
     _check(lib().snn_autotune_batch(hs, len(nets), int(trial_steps)))
@@ -257,7 +256,7 @@ def autotune_concurrent(nets, trial_steps: int = 200) -> list:
 
 
 def run_batch(nets, steps) -> None:
-    """Advance several networks together with one fused kernel per time step."""
+    """Advance several networks together in lockstep (see snn_run_batch)."""
     nets = list(nets)
     if isinstance(steps, int):
         steps = [steps] * len(nets)

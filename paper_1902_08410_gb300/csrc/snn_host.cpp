@@ -258,15 +258,15 @@ void build_inputs(const snn_params &p, BuildDev &bd) {
 // ---------------------------------------------------------------------------
 // network object
 // ---------------------------------------------------------------------------
-// Device arena of one network, in this order: V, c, ref, the input buffers of
-// the next min_delay + 1 steps, the spike counts and spike lists of the last
-// n_delay + min_delay steps (everything a run modifies), synapse rows, their
-// delay-group table, amplitude table, two windows, two recording blocks
+// Device arena of one network, in this order: V, c, ref, the spike counts of the
+// last n_delay + min_delay steps, 2 min_delay input buffers, the spike lists
+// (everything a run leaves behind), the persistent kernel's further input
+// buffers (zero between windows), synapse rows, their delay-group table, amplitude table, two windows, two recording blocks
 // (header, external-event slots, rate window: one contiguous copy per window),
 // two raster entry buffers.  Windows alternate between the two buffer sets, so
 // the host drains one window's records while the GPU runs the next.
 struct Layout {
-  size_t off_V, off_c, off_ref, off_acc, off_cnt, off_hist, off_rows, off_offs, off_amp;
+  size_t off_V, off_c, off_ref, off_cnt, off_acc, off_hist, off_more, off_rows, off_offs, off_amp;
   size_t off_win[2], off_rec[2], off_ext[2], off_rates[2], off_entries[2];
   size_t rec_block;   // bytes of one recording block
   size_t total;
@@ -336,9 +336,10 @@ static Layout make_layout(const snn_params &p) {
   L.off_V = take((size_t)L.N_pad * 4);
   L.off_c = take((size_t)L.N_pad * 4);
   L.off_ref = take((size_t)L.N_pad);
-  L.off_acc = take((size_t)L.nbuf * L.N_pad * 4);
   L.off_cnt = take((size_t)L.D * 4);
-  L.off_hist = take((size_t)L.D * L.N_pad * 4);
+  L.off_acc = take((size_t)L.nbuf * L.N_pad * 4);
+  L.off_hist = take((size_t)L.D * L.N_pad * 4);   // right behind acc: N_pad * 4 is a multiple of 256
+  L.off_more = take((size_t)kMaxVisit * L.N_pad * 4);
   L.off_rows = take((size_t)L.N * L.row_bytes);
   L.off_offs = take((size_t)L.N * L.os * 2);
   L.off_amp = take((size_t)kNPop * kZTab * 4);
@@ -442,7 +443,7 @@ static size_t l2_window_bytes(const snn_net *h) {
     cudaGetLastError();
     return 0;
   }
-  const size_t all = h->L.off_hist, state = h->L.off_acc;
+  const size_t all = h->L.off_hist, state = h->L.off_cnt;
   return std::min<size_t>(all <= g_l2_setaside ? all : state, (size_t)max_win);
 }
 
@@ -472,18 +473,32 @@ static int sm_count_cached() {
 // Delivery grid: deliver_blocks blocks per SM (every warp takes segments).
 static int deliver_grid(const snn_net *h);
 
+// The launch shape a network starts with leaves the form to the library: with
+// it, path 0 advances a window in one launch of the persistent kernel
+// (snn_run.cu).  A two-kernel shape set by the caller or chosen by a tuner is
+// run as two kernels per step.
+static void default_shape(snn_launch &c) {
+  c.update_block = 256;
+  c.deliver_warps = 16;
+  c.deliver_lanes = 32;
+  c.update_groups = 1;
+  c.deliver_blocks = 3;   // three 16-warp blocks per SM (40 registers)
+  c.overlap = 1;
+}
+
+static bool has_default_shape(const snn_launch &c) {
+  snn_launch d = c;
+  default_shape(d);
+  return std::memcmp(&d, &c, sizeof(c)) == 0;
+}
+
 static void default_launch(snn_net *h) {
+  default_shape(h->cfg);
   h->cfg.path = 0;
-  h->cfg.update_block = 256;
-  h->cfg.deliver_warps = 16;
   h->cfg.fused_block = 128;
   h->cfg.fused_items_per_sm = 8;
   h->cfg.window_steps = (int32_t)h->L.window;
-  h->cfg.deliver_lanes = 32;
-  h->cfg.update_groups = 1;
   h->cfg.l2_persist = 1;
-  h->cfg.deliver_blocks = 3;   // three 16-warp blocks per SM (40 registers)
-  h->cfg.overlap = 1;
 }
 
 extern "C" int snn_footprint(const snn_params *p, size_t *bytes_out) {
@@ -558,6 +573,10 @@ static void fill_descriptor(snn_net *h) {
     d.vr[q] = h->p.V_r[q];
     d.alpha[q] = h->p.alpha_c[q];
     d.narp[q] = t.narp;
+    float narp_bits;
+    std::memcpy(&narp_bits, &t.narp, 4);
+    d.pa[q] = make_float4(t.pvv, t.pvc, t.pcc, h->p.E_L[q]);
+    d.pb[q] = make_float4(h->p.V_th[q], h->p.V_r[q], h->p.alpha_c[q], narp_bits);
     for (int k = 0; k < kPoisMax; ++k) d.thr[q][k] = (uint32_t)t.thr[k];   // <= 2^20
   }
   d.V = reinterpret_cast<float *>(base + L.off_V);
@@ -608,6 +627,7 @@ extern "C" int snn_build_network(const snn_params *p, uint64_t seed, void *cuda_
   h->L = make_layout(*p);
   h->sm_count = sm_count_cached();
   CU_TRY(prepare_kernels());
+  CU_TRY(prepare_run_kernels());
   CU_TRY(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   CU_TRY(cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
   for (int b = 0; b < 2; ++b) CU_TRY(cudaEventCreateWithFlags(&h->ev_block[b], cudaEventDisableTiming));
@@ -656,7 +676,8 @@ extern "C" int snn_build_network(const snn_params *p, uint64_t seed, void *cuda_
   h->launches += 2;
   bd.cdf = d_cdf;
   bd.ztab = d_z;
-  CU_TRY(cudaMemsetAsync(base + L.off_acc, 0, L.off_hist - L.off_acc, s));   // inputs, spike counts
+  CU_TRY(cudaMemsetAsync(base + L.off_cnt, 0, L.off_hist - L.off_cnt, s));   // spike counts, inputs
+  CU_TRY(cudaMemsetAsync(base + L.off_more, 0, L.off_rows - L.off_more, s));
   CU_TRY(cudaMemsetAsync(base + L.off_win[0], 0, L.off_entries[0] - L.off_win[0], s));   // windows, blocks
   CU_TRY(cudaMallocHost(&h->pinned_win, 2 * sizeof(NetWin)));
   std::memset(h->pinned_win, 0, 2 * sizeof(NetWin));
@@ -788,6 +809,10 @@ static int drain_copy_entries(snn_net *h, int b, cudaStream_t s, uint32_t *n_out
     h->broken = true;
     return fail(SNN_ERR_LIMIT, "spike record window overflowed");
   }
+  if (rh->status & kStatusBarrier) {
+    h->broken = true;
+    return fail(SNN_ERR_CUDA, "a grid barrier of the run kernel was not met in time");
+  }
   const uint32_t n_rec = std::min(rh->cursor, L.rec_cap);
   if (n_rec) {
     if (h->pinned_entries_cap < n_rec) {
@@ -813,12 +838,18 @@ static int drain_absorb(snn_net *h, int b, uint64_t t0, uint32_t n_rec, cudaStre
   const unsigned long long *ext = reinterpret_cast<const unsigned long long *>(blk + (L.off_ext[b] - L.off_rec[b]));
   for (uint32_t i = 0; i < L.n_ext_slots; ++i) h->ext_events += ext[i];
   if (n_rec) {
+    // blocks record a step's spikes after they have met the others, so entries of neighbouring steps (of a whole
+    // exchange period) may come mixed: grouped by step here, the order within a step is left to the readers
     const size_t old = h->raster.size();
     h->raster.resize(old + n_rec);
+    std::vector<uint32_t> at(L.window + 1u, 0u);
+    for (uint32_t i = 0; i < n_rec; ++i) ++at[((h->pinned_entries[i] >> 32) & 0xFFFFu) + 1u];
+    for (uint32_t k = 0; k < L.window; ++k) at[k + 1u] += at[k];
+    unsigned long long *to = h->raster.data() + old;
     for (uint32_t i = 0; i < n_rec; ++i) {
       const unsigned long long e = h->pinned_entries[i];
       const uint64_t k = (e >> 32) & 0xFFFFu;
-      h->raster[old + i] = ((t0 + k) << 32) | (e & 0xFFFFFFFFull);
+      to[at[k]++] = ((t0 + k) << 32) | (e & 0xFFFFFFFFull);
     }
   }
   // rates of the window, bins from t0 / bin_steps
@@ -883,11 +914,19 @@ struct PlainRunner {
   snn_net *h = nullptr;
   uint32_t window = 0;
   uint64_t steps = 0, issued = 0, t_issue = 0;
+  RunShape shape;   // persistent kernel (blocks > 0), else two kernels per step
+  L2Window l2;
   Pending q[2];
   int nq = 0, next_b = 0;
   bool can_issue() const { return issued < steps && nq < 2; }
   bool busy() const { return issued < steps || nq > 0; }
 };
+
+static RunShape plain_shape(const snn_net *h) {
+  if (h->cfg.path == 0 && !has_default_shape(h->cfg)) return RunShape{};
+  const int threads = h->cfg.path == 1 ? h->cfg.fused_block * h->cfg.fused_items_per_sm : 1024;
+  return run_shape(h->L.N_pad / 128u, h->L.kmin, std::min(threads, 1024));
+}
 
 static uint32_t plain_window(const snn_net *h) {
   return (uint32_t)std::max(1, std::min<int32_t>(h->cfg.window_steps, (int32_t)h->L.window));
@@ -900,16 +939,33 @@ static int runner_issue(PlainRunner &r) {
   const uint64_t n = std::min<uint64_t>(r.window, r.steps - r.issued);
   if (t0 + n > 0xFFFFFFFFull) return fail(SNN_ERR_LIMIT, "step counter beyond 2^32");
   const int b = r.next_b;
-  NetWin *pw = h->pinned_win + b;   // free: the copy of its last use finished before that drain
-  set_window(h, pw, t0, t0 + n);
-  cudaGraphExec_t gx = nullptr;
-  uint32_t kernels = 0;
-  int rc = window_graph(h, b, (uint32_t)(t0 % h->L.nbuf), &gx, &kernels);
-  if (rc) return rc;
-  CU_TRY(cudaMemcpyAsync(base + h->L.off_win[b], pw, sizeof(NetWin), cudaMemcpyHostToDevice, h->stream));
-  CU_TRY(cudaGraphLaunch(gx, h->stream));
-  h->h2d += sizeof(NetWin);
-  h->launches += kernels;
+  int rc = SNN_OK;
+  if (r.shape.blocks > 0) {
+    RunArgs a{};
+    a.nd = descriptor(h, b);
+    set_window(h, &a.win, t0, t0 + n);
+    a.n_nets = 1;
+    a.n_tiles = h->L.N_pad / 128u;
+    a.steps = (uint32_t)n;
+    a.nd_max = (uint32_t)h->p.n_delay;
+    a.kmin = h->L.kmin;
+    // the barrier words follow the header in the recording block, which is zero at every window start
+    a.bar = reinterpret_cast<uint32_t *>(base + h->L.off_rec[b] + 128);
+    a.status = &a.nd.rec->status;
+    CU_TRY(launch_run(a, r.shape, r.l2, h->stream));
+    ++h->launches;
+  } else {
+    NetWin *pw = h->pinned_win + b;   // free: the copy of its last use finished before that drain
+    set_window(h, pw, t0, t0 + n);
+    cudaGraphExec_t gx = nullptr;
+    uint32_t kernels = 0;
+    rc = window_graph(h, b, (uint32_t)(t0 % h->L.nbuf), &gx, &kernels);
+    if (rc) return rc;
+    CU_TRY(cudaMemcpyAsync(base + h->L.off_win[b], pw, sizeof(NetWin), cudaMemcpyHostToDevice, h->stream));
+    CU_TRY(cudaGraphLaunch(gx, h->stream));
+    h->h2d += sizeof(NetWin);
+    h->launches += kernels;
+  }
   rc = drain_copy_block(h, b, h->stream);
   if (rc) return rc;
   r.q[r.nq++] = PlainRunner::Pending{b, t0, n};
@@ -928,13 +984,19 @@ static int runner_drain(PlainRunner &r) {
   return rc;
 }
 
-static int run_plain(snn_net *h, uint64_t steps) {
-  PlainRunner r;
+static int runner_start(PlainRunner &r, snn_net *h, uint64_t steps) {
   r.h = h;
   r.window = plain_window(h);
   r.steps = steps;
   r.t_issue = h->t;
-  int rc = prepare_graphs(h, r.window);
+  if (!steps) return SNN_OK;
+  r.shape = plain_shape(h);
+  return r.shape.blocks > 0 ? l2_window(h, &r.l2) : prepare_graphs(h, r.window);
+}
+
+static int run_plain(snn_net *h, uint64_t steps) {
+  PlainRunner r;
+  int rc = runner_start(r, h, steps);
   if (rc) return rc;
   int status = SNN_OK;
   while (status == SNN_OK && r.busy()) status = r.can_issue() ? runner_issue(r) : runner_drain(r);
@@ -948,14 +1010,8 @@ static int run_plain(snn_net *h, uint64_t steps) {
 static int run_plain_many(snn_net *const *hs, const uint64_t *steps, int32_t n) {
   std::vector<PlainRunner> rs((size_t)n);
   for (int i = 0; i < n; ++i) {
-    rs[i].h = hs[i];
-    rs[i].window = plain_window(hs[i]);
-    rs[i].steps = steps[i];
-    rs[i].t_issue = hs[i]->t;
-    if (steps[i]) {
-      int rc = prepare_graphs(hs[i], rs[i].window);
-      if (rc) return rc;
-    }
+    int rc = runner_start(rs[i], hs[i], steps[i]);
+    if (rc) return rc;
   }
   int status = SNN_OK;
   bool any = true;
@@ -973,164 +1029,85 @@ static int run_plain_many(snn_net *const *hs, const uint64_t *steps, int32_t n) 
 }
 
 // ---------------------------------------------------------------------------
-// fused path over a set of networks
+// lockstep runs of a set of networks
 // ---------------------------------------------------------------------------
+// Device tables of a batch, one set per calling thread (grown as needed, freed with the thread).
 struct BatchCtx {
-  DevBuf nets[2];              // NetDev[cap] per buffer set
-  DevBuf wins[2];              // NetWin[cap] per buffer set
-  DevBuf items;                // FusedItem[item_cap]
-  DevBuf n_items_dev;          // u32 item count read by the kernel
-  size_t cap = 0, item_cap = 0;
-  NetDev *pinned_nets = nullptr;   // [2][cap]
-  NetWin *pinned_wins = nullptr;   // [2][cap]
-  FusedItem *pinned_items = nullptr;
-  cudaStream_t cap_stream = nullptr, copy_stream = nullptr;
+  DevBuf tab[2];               // per buffer set: NetDev[cap], NetWin[cap], tile_pre[cap + 1], barrier words
+  size_t cap = 0;
+  uint8_t *pinned[2] = {nullptr, nullptr};
+  cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_block[2] = {nullptr, nullptr};
-  cudaGraphExec_t exec[2] = {nullptr, nullptr};
-  uint32_t exec_window = 0, exec_items = 0, exec_lanes = 0, exec_chunks = 0;
-  uint32_t pinned_count = 0;   // staging of the item count (copied before the replays)
-  int exec_block = 0, exec_blocks = 0;
-  void drop_graphs() {
-    for (auto &e : exec)
-      if (e) {
-        cudaGraphExecDestroy(e);
-        e = nullptr;
-      }
+  size_t wins_at() const { return cap * sizeof(NetDev); }
+  size_t pre_at() const { return wins_at() + cap * sizeof(NetWin); }
+  size_t bar_at() const { return align_up(pre_at() + (cap + 1) * 4, 256); }
+  size_t bytes() const { return bar_at() + 256; }
+  void drop() {
+    for (int b = 0; b < 2; ++b) {
+      tab[b].release();
+      if (pinned[b]) cudaFreeHost(pinned[b]);
+      pinned[b] = nullptr;
+    }
+    cap = 0;
   }
   ~BatchCtx() {
-    drop_graphs();
+    drop();
     for (auto e : ev_block)
       if (e) cudaEventDestroy(e);
-    if (cap_stream) cudaStreamDestroy(cap_stream);
     if (copy_stream) cudaStreamDestroy(copy_stream);
-    if (pinned_nets) cudaFreeHost(pinned_nets);
-    if (pinned_wins) cudaFreeHost(pinned_wins);
-    if (pinned_items) cudaFreeHost(pinned_items);
-    for (int b = 0; b < 2; ++b) {
-      nets[b].release();
-      wins[b].release();
-    }
-    items.release();
-    n_items_dev.release();
   }
 };
 static thread_local std::unique_ptr<BatchCtx> g_batch;
 
-static int run_fused(snn_net *const *hs, const uint64_t *steps, int32_t n) {
+// Networks of one smallest delay and one phase of its period advance in
+// lockstep, one launch of the persistent kernel per window; the table of a
+// window (descriptors, windows, tiles before each network, zeroed barrier
+// words) goes up in one copy.
+static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, const RunShape &shape, uint32_t n_tiles) {
   if (!g_batch) g_batch.reset(new BatchCtx());
   BatchCtx &B = *g_batch;
   const snn_launch &cfg = hs[0]->cfg;
-  const int block = cfg.fused_block;
-  const uint32_t npi = 4u * (uint32_t)block;
-  const uint32_t lanes = (uint32_t)cfg.deliver_lanes;
-  size_t n_items = 0;
-  uint32_t window = 0xFFFFFFFFu;
+  uint32_t window = 0xFFFFFFFFu, nd_max = 1;
   for (int i = 0; i < n; ++i) {
-    n_items += (hs[i]->L.N_pad + npi - 1) / npi;
     window = std::min<uint32_t>(window, hs[i]->L.window);
+    nd_max = std::max<uint32_t>(nd_max, (uint32_t)hs[i]->p.n_delay);
   }
   window = std::max<uint32_t>(1, std::min<uint32_t>(window, (uint32_t)std::max(1, cfg.window_steps)));
   if ((size_t)n > B.cap) {
-    for (int b = 0; b < 2; ++b) {
-      B.nets[b].release();
-      B.wins[b].release();
-    }
-    if (B.pinned_nets) cudaFreeHost(B.pinned_nets);
-    if (B.pinned_wins) cudaFreeHost(B.pinned_wins);
-    B.pinned_nets = nullptr;
-    B.pinned_wins = nullptr;
     const size_t cap = std::max<size_t>((size_t)n, 2 * B.cap);
-    B.cap = 0;
-    B.drop_graphs();
-    for (int b = 0; b < 2; ++b) {
-      int rc = dev_alloc(B.nets[b], cap * sizeof(NetDev));
-      if (rc) return rc;
-      rc = dev_alloc(B.wins[b], cap * sizeof(NetWin));
-      if (rc) return rc;
-    }
-    CU_TRY(cudaMallocHost(&B.pinned_nets, 2 * cap * sizeof(NetDev)));
-    CU_TRY(cudaMallocHost(&B.pinned_wins, 2 * cap * sizeof(NetWin)));
+    B.drop();
     B.cap = cap;
+    for (int b = 0; b < 2; ++b) {
+      int rc = dev_alloc(B.tab[b], B.bytes());
+      cudaError_t e = rc ? cudaSuccess : cudaMallocHost(&B.pinned[b], B.bytes());
+      if (rc || e != cudaSuccess) {
+        B.drop();
+        return rc ? rc : fail(SNN_ERR_OOM, std::string("cudaMallocHost: ") + cudaGetErrorString(e));
+      }
+    }
   }
-  if (n_items > B.item_cap) {
-    B.items.release();
-    if (B.pinned_items) cudaFreeHost(B.pinned_items);
-    B.pinned_items = nullptr;
-    const size_t cap = std::max<size_t>(n_items, 2 * B.item_cap);
-    B.item_cap = 0;
-    B.drop_graphs();
-    int rc = dev_alloc(B.items, cap * sizeof(FusedItem));
-    if (rc) return rc;
-    CU_TRY(cudaMallocHost(&B.pinned_items, cap * sizeof(FusedItem)));
-    B.item_cap = cap;
-  }
-  if (!B.cap_stream) CU_TRY(cudaStreamCreateWithFlags(&B.cap_stream, cudaStreamNonBlocking));
   if (!B.copy_stream) CU_TRY(cudaStreamCreateWithFlags(&B.copy_stream, cudaStreamNonBlocking));
   for (int b = 0; b < 2; ++b)
     if (!B.ev_block[b]) CU_TRY(cudaEventCreateWithFlags(&B.ev_block[b], cudaEventDisableTiming));
-  if (!B.n_items_dev.p) {
-    int rc = dev_alloc(B.n_items_dev, 256);
-    if (rc) return rc;
-  }
   cudaStream_t s = hs[0]->stream;
   // all networks of the batch are ordered on the first network's stream
+  bool other_streams = false;
   for (int i = 0; i < n; ++i)
-    if (hs[i]->stream != s) CU_TRY(cudaStreamSynchronize(hs[i]->stream));
-  size_t it = 0;
-  for (int i = 0; i < n; ++i) {
-    // items of network i: consecutive neuron ranges, each knowing its index
-    // among the network's items (its share of the network's delivery)
-    const uint32_t I = (hs[i]->L.N_pad + npi - 1) / npi;
-    for (uint32_t j = 0; j < I; ++j) B.pinned_items[it++] = FusedItem{(uint32_t)i, j * npi, j, I};
-  }
-  for (int b = 0; b < 2; ++b)
+    if (hs[i]->stream != s) {
+      other_streams = true;
+      CU_TRY(cudaStreamSynchronize(hs[i]->stream));
+    }
+  for (int b = 0; b < 2; ++b) {
+    uint32_t *pre = reinterpret_cast<uint32_t *>(B.pinned[b] + B.pre_at());
+    pre[0] = 0;
     for (int i = 0; i < n; ++i) {
       NetDev d = descriptor(hs[i], b);
       d.slot = (uint32_t)i;
-      d.win = static_cast<const NetWin *>(B.wins[b].p) + i;
-      B.pinned_nets[(size_t)b * B.cap + i] = d;
+      reinterpret_cast<NetDev *>(B.pinned[b])[i] = d;
+      pre[i + 1] = pre[i] + hs[i]->L.N_pad / 128u;
     }
-  uint32_t max_delay = 1;
-  for (int i = 0; i < n; ++i) max_delay = std::max<uint32_t>(max_delay, (uint32_t)hs[i]->p.n_delay);
-  const uint32_t chunks = pre_chunks(max_delay);   // delay chunks of the largest delay in the batch
-  const int sms = hs[0]->sm_count > 0 ? hs[0]->sm_count : 148;
-  const int per_sm = std::min(cfg.fused_items_per_sm, fused_blocks_per_sm(block, chunks));
-  const int blocks = sms * per_sm;   // fixed grid: the same graphs serve any set of networks
-  if (!B.exec[0] || !B.exec[1] || B.exec_window != window || B.exec_block != block || B.exec_blocks != blocks ||
-      B.exec_lanes != lanes || B.exec_chunks != chunks) {
-    B.drop_graphs();
-    for (int b = 0; b < 2; ++b) {
-      FusedTable tab{static_cast<const NetDev *>(B.nets[b].p), static_cast<const FusedItem *>(B.items.p),
-                     static_cast<const uint32_t *>(B.n_items_dev.p), lanes, chunks};
-      CU_TRY(cudaStreamBeginCapture(B.cap_stream, cudaStreamCaptureModeThreadLocal));
-      cudaError_t err = cudaSuccess;
-      for (uint32_t k = 0; k < window && err == cudaSuccess; ++k)
-        err = launch_fused(tab, k, block, blocks, B.cap_stream);
-      cudaGraph_t g = nullptr;
-      cudaError_t e2 = cudaStreamEndCapture(B.cap_stream, &g);
-      if (err != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return fail(SNN_ERR_CUDA, std::string("fused launch during capture: ") + cudaGetErrorString(err));
-      }
-      if (e2 != cudaSuccess) return fail(SNN_ERR_CUDA, std::string("end capture: ") + cudaGetErrorString(e2));
-      cudaError_t e3 = cudaGraphInstantiate(&B.exec[b], g, 0);
-      cudaGraphDestroy(g);
-      if (e3 != cudaSuccess) return fail(SNN_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e3));
-    }
-    B.exec_window = window;
-    B.exec_items = (uint32_t)n_items;
-    B.exec_block = block;
-    B.exec_blocks = blocks;
-    B.exec_lanes = lanes;
-    B.exec_chunks = chunks;
+    std::memset(B.pinned[b] + B.bar_at(), 0, 256);
   }
-  CU_TRY(cudaMemcpyAsync(B.items.p, B.pinned_items, n_items * sizeof(FusedItem), cudaMemcpyHostToDevice, s));
-  B.pinned_count = (uint32_t)n_items;
-  CU_TRY(cudaMemcpyAsync(B.n_items_dev.p, &B.pinned_count, 4, cudaMemcpyHostToDevice, s));
-  for (int b = 0; b < 2; ++b)
-    CU_TRY(cudaMemcpyAsync(B.nets[b].p, B.pinned_nets + (size_t)b * B.cap, (size_t)n * sizeof(NetDev),
-                           cudaMemcpyHostToDevice, s));
-  for (int i = 0; i < n; ++i) hs[i]->h2d += 2 * sizeof(NetDev);
 
   // windows alternate between the two buffer sets, two in flight at most
   struct Pending {
@@ -1147,7 +1124,7 @@ static int run_fused(snn_net *const *hs, const uint64_t *steps, int32_t n) {
     for (int i = 0; i < n; ++i) most = std::max(most, left[i]);
     if (most > 0 && nq < 2) {
       const int b = next_b;
-      NetWin *pw = B.pinned_wins + (size_t)b * B.cap;
+      NetWin *pw = reinterpret_cast<NetWin *>(B.pinned[b] + B.wins_at());   // free: its window has been drained
       Pending p{b, std::vector<uint64_t>(n), std::vector<uint64_t>(n)};
       for (int i = 0; i < n; ++i) {
         const uint64_t adv = std::min<uint64_t>(window, left[i]);
@@ -1160,11 +1137,25 @@ static int run_fused(snn_net *const *hs, const uint64_t *steps, int32_t n) {
         p.adv[i] = adv;
       }
       if (status != SNN_OK) break;
-      CU_TRY(cudaMemcpyAsync(B.wins[b].p, pw, (size_t)n * sizeof(NetWin), cudaMemcpyHostToDevice, s));
-      CU_TRY(cudaGraphLaunch(B.exec[b], s));
-      hs[0]->launches += window;   // one fused kernel per step for the whole batch
+      uint8_t *tab = static_cast<uint8_t *>(B.tab[b].p);
+      CU_TRY(cudaMemcpyAsync(tab, B.pinned[b], B.bytes(), cudaMemcpyHostToDevice, s));
+      RunArgs a{};
+      a.nets = reinterpret_cast<const NetDev *>(tab);
+      a.wins = reinterpret_cast<const NetWin *>(tab + B.wins_at());
+      a.tile_pre = reinterpret_cast<const uint32_t *>(tab + B.pre_at());
+      a.bar = reinterpret_cast<uint32_t *>(tab + B.bar_at());
+      a.n_nets = (uint32_t)n;
+      a.n_tiles = n_tiles;
+      a.steps = (uint32_t)std::min<uint64_t>(window, most);
+      a.nd_max = nd_max;
+      a.kmin = hs[0]->L.kmin;
+      int first = 0;   // a network that advances: its recording block is copied and checked
+      while (!p.adv[first]) ++first;
+      a.status = &reinterpret_cast<const NetDev *>(B.pinned[b])[first].rec->status;
+      CU_TRY(launch_run(a, shape, L2Window{}, s));
+      ++hs[0]->launches;
+      hs[0]->h2d += B.bytes();
       for (int i = 0; i < n; ++i) {
-        hs[i]->h2d += sizeof(NetWin);
         if (p.adv[i]) {
           int rc = drain_copy_block(hs[i], b, s);
           if (rc) return rc;
@@ -1185,8 +1176,48 @@ static int run_fused(snn_net *const *hs, const uint64_t *steps, int32_t n) {
     if (status == SNN_OK)
       for (int i = 0; i < n; ++i) hs[i]->t = p.t0s[i] + p.adv[i];
   }
-  if (status != SNN_OK) cudaStreamSynchronize(s);
+  // nothing left in flight; networks with a stream of their own may use it next
+  if (status != SNN_OK || other_streams) cudaStreamSynchronize(s);
   return status;
+}
+
+// A set of networks: grouped by smallest delay and phase, each group in as few
+// launches side by side as the blocks' shared memory allows.
+static int run_set(snn_net *const *hs, const uint64_t *steps, int32_t n) {
+  std::vector<int32_t> order(n);
+  for (int32_t i = 0; i < n; ++i) order[i] = i;
+  auto key = [&](int32_t i) { return std::make_pair(hs[i]->L.kmin, hs[i]->t % hs[i]->L.kmin); };
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return key(x) < key(y); });
+  const snn_launch &cfg = hs[0]->cfg;
+  const int threads = cfg.path == 1 ? std::min(1024, cfg.fused_block * cfg.fused_items_per_sm) : 1024;
+  for (int32_t at = 0; at < n;) {
+    std::vector<snn_net *> g;
+    std::vector<uint64_t> st;
+    RunShape shape;
+    uint64_t tiles = 0;
+    while (at < n && (g.empty() || key(order[at]) == std::make_pair(g[0]->L.kmin, g[0]->t % g[0]->L.kmin))) {
+      snn_net *h = hs[order[at]];
+      const RunShape next = run_shape((uint32_t)(tiles + h->L.N_pad / 128u), h->L.kmin, threads);
+      if (next.blocks < 1 && !g.empty()) break;
+      g.push_back(h);
+      st.push_back(steps[order[at]]);
+      tiles += h->L.N_pad / 128u;
+      shape = next;
+      ++at;
+      if (next.blocks < 1) break;   // too large for the persistent kernel by itself
+    }
+    const int rc = g.size() == 1 ? run_plain(g[0], st[0]) : run_lockstep(g.data(), st.data(), (int32_t)g.size(), shape, (uint32_t)tiles);
+    if (rc) return rc;
+  }
+  return SNN_OK;
+}
+
+// Networks of snn_run_concurrent: those that leave the form to the library
+// share one launch per window, else each runs on its own stream.
+static int run_together(snn_net *const *hs, const uint64_t *steps, int32_t n) {
+  bool together = n > 1;
+  for (int i = 0; i < n; ++i) together &= has_default_shape(hs[i]->cfg);
+  return together ? run_set(hs, steps, n) : run_plain_many(hs, steps, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -1196,10 +1227,6 @@ extern "C" int snn_run(snn_handle h, uint64_t steps) {
   if (!h) return fail(SNN_ERR_ARG, "null handle");
   if (h->broken) return fail(SNN_ERR_STATE, "network is invalid after an earlier failure");
   if (steps == 0) return SNN_OK;
-  if (h->cfg.path == 1) {
-    snn_net *one[1] = {h};
-    return run_fused(one, &steps, 1);
-  }
   return run_plain(h, steps);
 }
 
@@ -1212,7 +1239,7 @@ extern "C" int snn_run_batch(const snn_handle *hs, const uint64_t *steps, int32_
     for (int j = 0; j < i; ++j)
       if (hs[j] == hs[i]) return fail(SNN_ERR_ARG, "a network appears twice in the batch");
   }
-  return run_fused(hs, steps, n);
+  return run_set(hs, steps, n);
 }
 
 extern "C" int snn_run_concurrent(const snn_handle *hs, const uint64_t *steps, int32_t n) {
@@ -1221,11 +1248,11 @@ extern "C" int snn_run_concurrent(const snn_handle *hs, const uint64_t *steps, i
   for (int i = 0; i < n; ++i) {
     if (!hs[i]) return fail(SNN_ERR_ARG, "null handle");
     if (hs[i]->broken) return fail(SNN_ERR_STATE, "network is invalid after an earlier failure");
-    if (hs[i]->cfg.path != 0) return fail(SNN_ERR_ARG, "snn_run_concurrent runs the two-kernel path (launch path 0)");
+    if (hs[i]->cfg.path != 0) return fail(SNN_ERR_ARG, "snn_run_concurrent runs launch path 0");
     for (int j = 0; j < i; ++j)
       if (hs[j] == hs[i]) return fail(SNN_ERR_ARG, "a network appears twice");
   }
-  return run_plain_many(hs, steps, n);
+  return run_together(hs, steps, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -1351,19 +1378,19 @@ extern "C" int snn_time_kernels(snn_handle h, uint32_t steps, double *ms_out) {
   if (rc) return rc;
   rc = capture_steps(h, descriptor(h, 0), steps, phase, l2, ev.data(), &guard.gx[1], nullptr);
   if (rc) return rc;
-  rc = dev_alloc(guard.snap, L.off_rows);   // V, c, ref, input buffers, spike history
+  rc = dev_alloc(guard.snap, L.off_more);   // V, c, ref, input buffers, spike history
   if (rc) return rc;
   set_window(h, h->pinned_win, t0, t0 + steps);
   CU_TRY(cudaMemcpyAsync(base + L.off_win[0], h->pinned_win, sizeof(NetWin), cudaMemcpyHostToDevice, s));
   // (1) the steps as snn_run runs them, from a snapshot that is restored after
-  CU_TRY(cudaMemcpyAsync(guard.snap.p, base, L.off_rows, cudaMemcpyDeviceToDevice, s));
+  CU_TRY(cudaMemcpyAsync(guard.snap.p, base, L.off_more, cudaMemcpyDeviceToDevice, s));
   cudaEvent_t a = ev[4 * (size_t)steps], b = ev[4 * (size_t)steps + 1];
   CU_TRY(cudaGraphUpload(guard.gx[0], s));   // keep the first launch's upload out of the timed span
   CU_TRY(cudaGraphUpload(guard.gx[1], s));
   CU_TRY(cudaEventRecord(a, s));
   CU_TRY(cudaGraphLaunch(guard.gx[0], s));
   CU_TRY(cudaEventRecord(b, s));
-  CU_TRY(cudaMemcpyAsync(base, guard.snap.p, L.off_rows, cudaMemcpyDeviceToDevice, s));
+  CU_TRY(cudaMemcpyAsync(base, guard.snap.p, L.off_more, cudaMemcpyDeviceToDevice, s));
   CU_TRY(cudaMemsetAsync(base + L.off_rec[0], 0, L.rec_block, s));
   // (2) the same steps with event nodes around every kernel; these results stay
   CU_TRY(cudaGraphLaunch(guard.gx[1], s));
@@ -1392,7 +1419,7 @@ extern "C" int snn_time_kernels(snn_handle h, uint32_t steps, double *ms_out) {
 }
 
 // ---------------------------------------------------------------------------
-// batch tuner: fused-kernel shapes timed on the whole batch from snapshots of
+// batch tuner: path 1 shapes timed on the whole batch from snapshots of
 // every network, restored after each trial
 // ---------------------------------------------------------------------------
 // Snapshots of several networks for the multi-network tuners: state (V, c,
@@ -1424,9 +1451,9 @@ struct MultiSnapshot {
     sv.resize((size_t)n);
     for (int i = 0; i < n; ++i) {
       snn_net *h = hs[i];
-      int rc = dev_alloc(sv[i].snap, h->L.off_rows);   // V, c, ref, input buffers, spike history
+      int rc = dev_alloc(sv[i].snap, h->L.off_more);   // V, c, ref, input buffers, spike history
       if (rc) return rc;
-      CU_TRY(cudaMemcpyAsync(sv[i].snap.p, h->arena.p, h->L.off_rows, cudaMemcpyDeviceToDevice, s));
+      CU_TRY(cudaMemcpyAsync(sv[i].snap.p, h->arena.p, h->L.off_more, cudaMemcpyDeviceToDevice, s));
       sv[i].t = h->t;
       sv[i].spikes = h->spikes;
       sv[i].ext = h->ext_events;
@@ -1441,7 +1468,7 @@ struct MultiSnapshot {
     for (int i = 0; i < n; ++i) {
       snn_net *h = hs[i];
       uint8_t *base = static_cast<uint8_t *>(h->arena.p);
-      CU_TRY(cudaMemcpyAsync(base, sv[i].snap.p, h->L.off_rows, cudaMemcpyDeviceToDevice, s));
+      CU_TRY(cudaMemcpyAsync(base, sv[i].snap.p, h->L.off_more, cudaMemcpyDeviceToDevice, s));
       CU_TRY(cudaMemsetAsync(base + h->L.off_rec[0], 0, h->L.off_entries[0] - h->L.off_rec[0], s));   // both blocks
       h->t = sv[i].t;
       h->spikes = sv[i].spikes;
@@ -1488,7 +1515,7 @@ extern "C" int snn_autotune_batch(const snn_handle *hs, int32_t n, uint32_t tria
       int r = snap.restore();
       if (r) return r;
       CU_TRY(cudaEventRecord(e0, s));
-      r = run_fused(hs, steps.data(), n);
+      r = run_set(hs, steps.data(), n);
       if (r) return r;
       CU_TRY(cudaEventRecord(e1, s));
       CU_TRY(cudaEventSynchronize(e1));
@@ -1503,21 +1530,18 @@ extern "C" int snn_autotune_batch(const snn_handle *hs, int32_t n, uint32_t tria
   float orig_ms = 1e30f, best_ms = 1e30f;
   snn_launch best = orig;
   int status = trial(orig, 2, &orig_ms);
-  for (int fb : {128, 256, 512})
-    for (int ips : {2, 4, 8, 16})
-      for (int ln : {8, 16, 32}) {
-        if (status != SNN_OK) break;
-        snn_launch c = orig;
-        c.fused_block = fb;
-        c.fused_items_per_sm = ips;
-        c.deliver_lanes = ln;
-        float ms = 0;
-        status = trial(c, 1, &ms);
-        if (status == SNN_OK && ms < best_ms) {
-          best_ms = ms;
-          best = c;
-        }
-      }
+  for (int ips : {2, 4, 6, 8}) {   // 256 .. 1024 threads per SM
+    if (status != SNN_OK) break;
+    snn_launch c = orig;
+    c.fused_block = 128;
+    c.fused_items_per_sm = ips;
+    float ms = 0;
+    status = trial(c, 1, &ms);
+    if (status == SNN_OK && ms < best_ms) {
+      best_ms = ms;
+      best = c;
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   int rr = snap.restore();
@@ -1530,7 +1554,7 @@ extern "C" int snn_autotune_concurrent(const snn_handle *hs, int32_t n, uint32_t
   int rc = check_multi(hs, n, trial_steps, 1024);
   if (rc) return rc;
   for (int i = 0; i < n; ++i)
-    if (hs[i]->cfg.path != 0) return fail(SNN_ERR_ARG, "snn_autotune_concurrent tunes the two-kernel path (launch path 0)");
+    if (hs[i]->cfg.path != 0) return fail(SNN_ERR_ARG, "snn_autotune_concurrent tunes launch path 0");
   MultiSnapshot snap;
   rc = snap.take(hs, n);
   if (rc) return rc;
@@ -1555,7 +1579,7 @@ extern "C" int snn_autotune_concurrent(const snn_handle *hs, int32_t n, uint32_t
       if (r) return r;
       CU_TRY(cudaEventRecord(ev[0], hs[0]->stream));
       for (int i = 1; i < n; ++i) CU_TRY(cudaStreamWaitEvent(hs[i]->stream, ev[0], 0));
-      r = run_plain_many(hs, steps.data(), n);
+      r = run_together(hs, steps.data(), n);
       if (r) return r;
       for (int i = 0; i < n; ++i) CU_TRY(cudaEventRecord(ev[(size_t)i + 1], hs[i]->stream));
       float ms = 0;
@@ -1650,7 +1674,7 @@ extern "C" int snn_set_launch(snn_handle h, const snn_launch *cfg) {
 // autotuner: time candidate shapes from a snapshot of the state, restore the
 // snapshot after each trial, so the network's results are unchanged.
 // ---------------------------------------------------------------------------
-// path_only: -1 = both launch paths, 0 = two-kernel path only, 1 = fused only.
+// path_only: -1 = both launch paths, 0 = path 0 only, 1 = path 1 only.
 static int autotune_impl(snn_net *h, uint32_t trial_steps, int path_only) {
   if (!h) return fail(SNN_ERR_ARG, "null handle");
   if (h->broken) return fail(SNN_ERR_STATE, "network is invalid after an earlier failure");
@@ -1658,7 +1682,7 @@ static int autotune_impl(snn_net *h, uint32_t trial_steps, int path_only) {
   if (path_only < -1 || path_only > 1) return fail(SNN_ERR_ARG, "path must be -1, 0 or 1");
   const Layout &L = h->L;
   uint8_t *base = static_cast<uint8_t *>(h->arena.p);
-  const size_t state_bytes = L.off_rows;   // V, c, ref, input buffers, spike history
+  const size_t state_bytes = L.off_more;   // V, c, ref, input buffers, spike history
   DevBuf snap;
   int rc = dev_alloc(snap, state_bytes);
   if (rc) return rc;
@@ -1679,7 +1703,7 @@ static int autotune_impl(snn_net *h, uint32_t trial_steps, int path_only) {
   snn_launch orig = h->cfg;   // the incumbent, on the allowed path
   if (path_only >= 0) orig.path = path_only;
 
-  // stage 1: update shapes with the current delivery shape, and the fused path
+  // stage 1: update shapes with the current delivery shape, and path 1
   std::vector<snn_launch> cands;
   for (int ub : {64, 128, 256})
     for (int ug : {1, 2, 4}) {
@@ -1691,17 +1715,14 @@ static int autotune_impl(snn_net *h, uint32_t trial_steps, int path_only) {
       c.update_groups = ug;
       cands.push_back(c);
     }
-  for (int fb : {128, 256})
-    for (int ips : {4, 8, 16})
-      for (int ln : {8, 16}) {
-        if (path_only == 0) continue;
-        snn_launch c = orig;
-        c.path = 1;
-        c.fused_block = fb;
-        c.fused_items_per_sm = ips;
-        c.deliver_lanes = ln;
-        cands.push_back(c);
-      }
+  for (int ips : {4, 8}) {
+    if (path_only == 0) continue;
+    snn_launch c = orig;
+    c.path = 1;
+    c.fused_block = 128;
+    c.fused_items_per_sm = ips;
+    cands.push_back(c);
+  }
   cudaEvent_t e0, e1;
   CU_TRY(cudaEventCreate(&e0));
   CU_TRY(cudaEventCreate(&e1));

@@ -17,6 +17,7 @@ constexpr int kNeuronAlign = 128; // neuron arrays padded to a multiple of 128
 
 // status bits written by kernels
 constexpr uint32_t kStatusRasterOverflow = 2u;
+constexpr uint32_t kStatusBarrier = 4u;   // a grid barrier ran out of its polling limit
 
 // Time window of one graph replay (device memory, rewritten by the host
 // before every replay so that captured graphs stay valid).
@@ -41,14 +42,15 @@ struct StepMod {
 };
 
 // Recording header of a network (device memory, zeroed at every window start).
+// The barrier words of the persistent kernel lie 128 bytes behind it.
 struct alignas(16) RecHeader {
   uint32_t cursor;        // raster entries appended in this window
   uint32_t status;        // kStatus* bits
   uint32_t pad[2];
 };
 
-// Static description of a network.  Passed by value as a kernel parameter on
-// the single-network path and stored in a device table on the fused path.
+// Static description of a network.  Passed by value as a kernel parameter for
+// a single network and stored in a device table for several.
 struct alignas(16) NetDev {
   // --- sizes
   uint32_t N;           // neurons
@@ -75,7 +77,10 @@ struct alignas(16) NetDev {
   float el[kNPop], vth[kNPop], vr[kNPop], alpha[kNPop];
   int32_t narp[kNPop];
   uint32_t pad0[2];
-  uint32_t thr[kNPop][kPoisMax];   // Poisson CDF thresholds, scaled by 2^20
+  alignas(16) uint32_t thr[kNPop][kPoisMax];   // Poisson CDF thresholds, scaled by 2^20 (read four at a time)
+  // the same constants as two 16-byte loads per population: {pvv, pvc, pcc, el}
+  // and {vth, vr, alpha, narp (bits)}
+  float4 pa[kNPop], pb[kNPop];
 
   // --- device arrays
   float *V;             // [N_pad]
@@ -83,7 +88,8 @@ struct alignas(16) NetDev {
   uint8_t *ref;         // [N_pad]
   // Synaptic input of step t (2^-16 mV): acc[t % nbuf][n], accumulated by
   // reductions during the delivery pass before step t, cleared by the update.
-  int32_t *acc;         // [nbuf][N_pad]
+  // The persistent kernel has kMaxVisit more behind hist, zero between windows.
+  int32_t *acc;         // [nbuf][N_pad], directly followed by hist
   uint32_t *cnt;        // [D] spikes of the step with slot t mod D
   uint32_t *hist;       // [D][N_pad] their ids, in the order they were appended
   uint8_t *rows;        // [N][row_bytes]
@@ -96,6 +102,10 @@ struct alignas(16) NetDev {
   unsigned long long *ext_acc;      // [N_pad / 128] external events per 128-neuron group
 };
 
+static_assert(offsetof(NetDev, thr) % 16 == 0 && offsetof(NetDev, pa) % 16 == 0 && offsetof(NetDev, pb) % 16 == 0 &&
+                  sizeof(NetDev) % 16 == 0 && sizeof(NetWin) % 16 == 0,
+              "16-byte loads of the descriptor tables");
+
 // Construction-time inputs.
 struct BuildDev {
   const uint32_t *cdf;  // [G][G-1] module thresholds
@@ -105,24 +115,6 @@ struct BuildDev {
   uint32_t n_delay;     // delays uniform on min_delay..n_delay
   uint32_t min_delay;
   int32_t p_local_mode; // 1 when p_local >= 0 (local bucket shortcut valid), 0 otherwise
-};
-
-// Work item of the fused step kernel: a range of one network's neurons to
-// update; the item's index among its network's items also selects its share
-// of the network's delivery work.
-struct FusedItem {
-  uint32_t net;         // index into the NetDev table
-  uint32_t n_begin;     // first neuron (multiple of 4)
-  uint32_t index;       // index of the item among its network's items
-  uint32_t count;       // items of the network
-};
-
-struct FusedTable {
-  const NetDev *nets;
-  const FusedItem *items;
-  const uint32_t *n_items;  // item count in device memory (the graph outlives any one batch)
-  uint32_t lanes;           // lanes per delivery segment
-  uint32_t chunks;          // register prefix chunks of 32 delays: 1 or kMaxPreChunks (largest n_delay of the table)
 };
 
 // ---- launchers (snn_kernels.cu) -------------------------------------------
@@ -140,8 +132,42 @@ cudaError_t launch_update(const NetDev &nd, uint32_t k, StepMod km, int block, i
                           bool pdl, cudaStream_t s);
 cudaError_t launch_deliver(const NetDev &nd, uint32_t k, StepMod km, uint32_t lanes, int warps, int blocks,
                            const L2Window &l2, bool pdl, cudaStream_t s);
-cudaError_t launch_fused(const FusedTable &tab, uint32_t k, int block, int blocks, cudaStream_t s);
-int fused_blocks_per_sm(int block, uint32_t chunks);   // resident fused blocks per SM
+
+// Persistent kernel: steps between two visits of a live spike, at most; kmin = 1
+// networks have visit + 2 input buffers.
+constexpr uint32_t kMaxVisit = 4;
+
+// Persistent kernel: a window of steps of one or more networks in one launch
+// (snn_run.cu).
+struct RunArgs {
+  NetDev nd;                  // single network: its descriptor and window
+  NetWin win;
+  const NetDev *nets;         // several networks: device tables [n_nets]
+  const NetWin *wins;
+  const uint32_t *tile_pre;   // [n_nets + 1] 128-neuron tiles before each network
+  uint32_t n_nets;
+  uint32_t n_tiles;           // tiles of all networks
+  uint32_t steps;             // steps of the window (the longest of the networks)
+  uint32_t nd_max;            // largest delay of the networks
+  uint32_t kmin;              // smallest delay, the same for all networks
+  uint32_t visit;             // steps between two visits of a live spike (1 in the period form)
+  uint32_t fifo;              // live spikes of one ring that a block holds in shared memory (power of two)
+  uint32_t nt;                // tiles of a block, at most
+  uint32_t pre;               // records of a new spike's row prefetched (multiple of 8)
+  // {grid barrier count, last step (+1) that overflowed a live list, lists not taken over}, zero at launch
+  uint32_t *bar;
+  uint32_t *status;           // status word of a network that advances
+};
+struct RunShape {
+  int blocks = 0, threads = 0;
+  int form = 0;               // RunForm
+  uint32_t fifo = 0, nt = 0, visit = 1;
+  size_t smem = 0;
+};
+// blocks == 0: too many tiles for one launch.
+RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads);
+cudaError_t launch_run(const RunArgs &a, const RunShape &sh, const L2Window &l2, cudaStream_t s);
+cudaError_t prepare_run_kernels();
 // Delivery keeps each warp's segment prefix in registers, in chunks of 32
 // delays: one chunk up to n_delay 32, else kMaxPreChunks (n_delay <= 256).
 constexpr uint32_t kMaxPreChunks = 8;

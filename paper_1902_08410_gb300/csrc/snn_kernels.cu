@@ -31,226 +31,10 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "snn_device.cuh"
 #include "snn_internal.h"
 
 namespace snn {
-
-// ---------------------------------------------------------------------------
-// Philox4x32-10 (Salmon et al., SC'11): ten rounds, Weyl key schedule.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                               uint32_t k0, uint32_t k1) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t lo0 = 0xD2511F53u * c0;
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c0);
-    const uint32_t lo1 = 0xCD9E8D57u * c2;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2);
-    const uint32_t n0 = hi1 ^ c1 ^ k0;
-    const uint32_t n2 = hi0 ^ c3 ^ k1;
-    c0 = n0;
-    c1 = lo1;
-    c2 = n2;
-    c3 = lo0;
-    k0 += 0x9E3779B9u;
-    k1 += 0xBB67AE85u;
-  }
-  return make_uint4(c0, c1, c2, c3);
-}
-
-__device__ __forceinline__ int pop_of_local(uint32_t local) { return local < 250u ? 0 : (local < 1000u ? 1 : 2); }
-
-__device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
-
-// Fire-and-forget prefetch of [src, src + bytes) into L2 (16-byte aligned
-// address, size a multiple of 16).
-__device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
-// Prefetch the byte range [p, p + bytes) widened to 16-byte boundaries; the
-// caller guarantees the widened range lies inside one allocation.
-__device__ __forceinline__ void prefetch_range_l2(const uint8_t *p, uint32_t bytes) {
-  if (bytes == 0) return;
-  const uintptr_t a0 = reinterpret_cast<uintptr_t>(p) & ~uintptr_t(15);
-  const uintptr_t a1 = (reinterpret_cast<uintptr_t>(p) + bytes + 15u) & ~uintptr_t(15);
-  bulk_prefetch_l2(reinterpret_cast<const void *>(a0), (uint32_t)(a1 - a0));
-}
-
-// Programmatic dependent launch: wait for the previous kernel in the stream
-// (no-op when launched without the attribute), then let the next one launch.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// ---------------------------------------------------------------------------
-// Fire-and-forget global reductions (no value returned, no scoreboard wait).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void red_add_s32(int32_t *addr, int32_t v) {
-  asm volatile("red.relaxed.gpu.global.add.s32 [%0], %1;" ::"l"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void red_add_u32(uint32_t *addr, uint32_t v) {
-  asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void red_add_u64(unsigned long long *addr, unsigned long long v) {
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(addr), "l"(v) : "memory");
-}
-
-// L2-only loads (never served from L1) of data that other kernels of the
-// stream write: the neuron state and input buffers, and the spike lists and
-// counts, which the update of a step appends to while an overlapping delivery
-// pass reads older slots of the same arrays.  L1 stays for the amplitude table.
-__device__ __forceinline__ float4 ld_cg_f4(const float4 *p) {
-  float4 v;
-  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "l"(p));
-  return v;
-}
-__device__ __forceinline__ int4 ld_cg_i4(const int4 *p) {
-  int4 v;
-  asm volatile("ld.global.cg.v4.s32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-__device__ __forceinline__ uint32_t ld_cg_u32(const uint32_t *p) {
-  uint32_t v;
-  asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p));
-  return v;
-}
-// Read-only loads of synapse records, not kept in L1 (each is used once).
-__device__ __forceinline__ uint32_t ld_rec_u32(const uint32_t *p) {
-  uint32_t v;
-  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ float ld_rec_f32(const float *p) {
-  float v;
-  asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ int32_t ld_rec_s16(const int16_t *p) {
-  int16_t v;
-  asm volatile("ld.global.nc.L1::no_allocate.s16 %0, [%1];" : "=h"(v) : "l"(p));
-  return (int32_t)v;
-}
-
-// ---------------------------------------------------------------------------
-// Neuron update (Eq. 2 over one step, Poisson drive) of 4 consecutive neurons.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t poisson_count(const NetDev &nd, int pop, uint32_t w) {
-  const uint32_t u = w >> 12;   // 20-bit uniform
-  uint32_t k = 0;
-  while (k < (uint32_t)kPoisMax && u >= nd.thr[pop][k]) ++k;
-  return k;
-}
-
-// Amplitudes of external events e0..k-1 of neuron n at step t (2^-16 mV), one
-// Philox draw per 8 events; only the rare tail e0 = 9 comes through here.
-__device__ __noinline__ int32_t extra_amplitudes(const NetDev &nd, int pop, uint32_t e0, uint32_t k, uint32_t n,
-                                                 uint32_t t) {
-  const int32_t *ap = nd.amp + pop * kZTab;
-  int32_t I = 0;
-  uint4 q = make_uint4(0, 0, 0, 0);
-  for (uint32_t e = e0; e < k; ++e) {
-    const uint32_t i = (e - 1u) & 7u;
-    if (e == e0 || i == 0) q = philox4x32_10(n, t, 3u, (e - 1u) >> 3, nd.key0, nd.key1);
-    const uint32_t w = i >> 1;
-    const uint32_t word = (w == 0) ? q.x : ((w == 1) ? q.y : ((w == 2) ? q.z : q.w));
-    const uint32_t half = (i & 1u) ? (word >> 16) : (word & 0xFFFFu);
-    I += __ldg(ap + (half >> 4));
-  }
-  return I;
-}
-
-// Amplitudes of events 1..k-1 (k >= 2) of neuron n: events 1..8 come from the
-// halves of one draw and their table loads are independent.
-__device__ __forceinline__ int32_t extra_sum(const NetDev &nd, int pop, uint32_t k, uint32_t n, uint32_t t) {
-  const int32_t *ap = nd.amp + pop * kZTab;
-  const uint4 R = philox4x32_10(n, t, 3u, 0u, nd.key0, nd.key1);
-  const uint32_t h[8] = {R.x & 0xFFFFu, R.x >> 16, R.y & 0xFFFFu, R.y >> 16,
-                         R.z & 0xFFFFu, R.z >> 16, R.w & 0xFFFFu, R.w >> 16};
-  int32_t I = 0;
-#pragma unroll
-  for (uint32_t j = 0; j < 8u; ++j)
-    if (j + 1u < k) I += __ldg(ap + (h[j] >> 4));
-  if (k > 9u) I += extra_amplitudes(nd, pop, 9u, k, n, t);
-  return I;
-}
-
-// Events 1..k-1 of every neuron of the warp's 128-neuron tile that received
-// more than one external event this step (about 1.4% of neurons at 0.18
-// expected events).  The pending (lane, q) pairs are numbered q-major by
-// ballots and lane i serves pair i, so a warp pays one draw and one table
-// round trip instead of one per neuron and event; sums return by shuffle.
-// Called by whole warps (all 32 lanes).
-__device__ __forceinline__ void extra_events_warp(const NetDev &nd, uint32_t n0, uint32_t t, const uint32_t (&kx)[4],
-                                                  int32_t (&Iv)[4]) {
-  if (!__any_sync(0xFFFFFFFFu, kx[0] > 1u || kx[1] > 1u || kx[2] > 1u || kx[3] > 1u)) return;   // most warps
-  const uint32_t lane = lane_id(), lt = (1u << lane) - 1u;
-  uint32_t bal[4], idx[4], cnt[4], total = 0;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    bal[q] = __ballot_sync(0xFFFFFFFFu, kx[q] > 1u);
-    idx[q] = total + __popc(bal[q] & lt);
-    cnt[q] = total;
-    total += __popc(bal[q]);
-  }
-  if (total == 0u) return;
-  const uint32_t packed = kx[0] | (kx[1] << 8) | (kx[2] << 16) | (kx[3] << 24);   // each count <= 16
-  const uint32_t tile0 = n0 - lane * 4u;
-  for (uint32_t s = 0; s < total; s += 32u) {
-    const uint32_t i = s + lane;
-    uint32_t q = 0, owner = 0;
-    if (i < total) {
-      q = (i >= cnt[1] ? 1u : 0u) + (i >= cnt[2] ? 1u : 0u) + (i >= cnt[3] ? 1u : 0u);
-      uint32_t b = (q == 0u) ? bal[0] : ((q == 1u) ? bal[1] : ((q == 2u) ? bal[2] : bal[3]));
-      const uint32_t base = (q == 0u) ? 0u : ((q == 1u) ? cnt[1] : ((q == 2u) ? cnt[2] : cnt[3]));
-      for (uint32_t r = base; r < i; ++r) b &= b - 1u;   // drop the lower set bits: rank i - base
-      owner = (uint32_t)(__ffs(b) - 1);
-    }
-    const uint32_t pk = __shfl_sync(0xFFFFFFFFu, packed, owner);
-    int32_t acc = 0;
-    if (i < total) {
-      const uint32_t n = tile0 + owner * 4u + q;
-      acc = extra_sum(nd, pop_of_local(n % (uint32_t)kK), (pk >> (8u * q)) & 0xFFu, n, t);
-    }
-#pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-      const int32_t v = __shfl_sync(0xFFFFFFFFu, acc, idx[qq] & 31u);
-      if (kx[qq] > 1u && idx[qq] - s < 32u) Iv[qq] += v;
-    }
-  }
-}
-
-
-__device__ __forceinline__ bool neuron_step(const NetDev &nd, int pop, float &V, float &c, uint32_t &ref, int32_t I) {
-  bool spike = false;
-  const float c_old = c;
-  if (ref > 0u) {
-    ref -= 1u;
-    V = nd.vr[pop];
-  } else {
-    const float el = nd.el[pop];
-    const float a = __fsub_rn(V, el);
-    const float b = __fmul_rn(nd.pvv[pop], a);
-    const float e = __fmul_rn(nd.pvc[pop], c_old);
-    const float f = __fadd_rn(b, e);
-    const float g = __fadd_rn(el, f);
-    const float x = __fmul_rn(__int2float_rn(I), 1.0f / 65536.0f);
-    float vn = __fadd_rn(g, x);
-    if (vn > nd.vth[pop]) {
-      spike = true;
-      vn = nd.vr[pop];
-      ref = (uint32_t)nd.narp[pop];
-    }
-    V = vn;
-  }
-  float cn = __fmul_rn(nd.pcc[pop], c_old);
-  if (spike) cn = __fadd_rn(cn, nd.alpha[pop]);
-  c = cn;
-  return spike;
-}
 
 // State of 4 consecutive neurons n0..n0+3 (n0 % 4 == 0, n0 < N_pad).
 struct Group4 {
@@ -325,17 +109,6 @@ __device__ __forceinline__ uint32_t integrate4(const NetDev &nd, uint32_t n0, ui
   return mask;
 }
 
-// One step of 4 neurons: the state and input loads are issued first and are
-// in flight while the drive is computed.
-__device__ __forceinline__ uint32_t update4(const NetDev &nd, uint32_t n0, uint32_t t, uint32_t buf, uint32_t &n_ext) {
-  Group4 g;
-  load_state4(nd, n0, g);
-  load_input4(nd, n0, buf, g);
-  int32_t I[4] = {0, 0, 0, 0};
-  drive4(nd, n0, t, I, n_ext);
-  return integrate4(nd, n0, buf, g, I);
-}
-
 // Slot (t mod D) of step t = t0 + k from the window's residue and the step's,
 // without a division.
 __device__ __forceinline__ uint32_t step_slot(const NetDev &nd, const NetWin &w, StepMod km) {
@@ -349,12 +122,11 @@ __device__ __forceinline__ uint32_t step_slot(const NetDev &nd, const NetWin &w,
 // step's spike list (`hist`) with one returning atomic each per warp, counts
 // rates with fire-and-forget reductions, adds each tile's external events to
 // that tile's slot and prefetches into L2 the delay-group table and the first
-// records of every spiking neuron's row.  When `smem_list` is given the ids
-// are also appended there (block-local list for the fused step).
+// records of every spiking neuron's row.
 template <int G>
 __device__ __forceinline__ void record_warp(const NetDev &nd, const uint32_t (&mask)[G], const uint32_t (&n0)[G],
                                             const uint32_t (&n_ext)[G], uint32_t t, uint32_t slot, uint32_t k,
-                                            uint32_t bin0, uint32_t *smem_list, uint32_t *smem_count) {
+                                            uint32_t bin0) {
   const uint32_t lane = lane_id();
   const uint32_t lt = (1u << lane) - 1u;
   uint32_t before[G], wtot = 0;
@@ -374,15 +146,13 @@ __device__ __forceinline__ void record_warp(const NetDev &nd, const uint32_t (&m
     if (lane == 0 && ext) red_add_u64(nd.ext_acc + tile, ext);   // slot owned by this warp
   }
   if (wtot == 0) return;
-  uint32_t gbase = 0, hbase = 0, sbase = 0;
+  uint32_t gbase = 0, hbase = 0;
   if (lane == 0) {
     gbase = atomicAdd(&nd.rec->cursor, wtot);
     hbase = atomicAdd(nd.cnt + slot, wtot);
-    if (smem_list) sbase = atomicAdd(smem_count, wtot);
   }
   gbase = __shfl_sync(0xFFFFFFFFu, gbase, 0);
   hbase = __shfl_sync(0xFFFFFFFFu, hbase, 0);
-  sbase = __shfl_sync(0xFFFFFFFFu, sbase, 0);
   if (lane == 0 && gbase + wtot > nd.rec_cap) atomicOr(&nd.rec->status, kStatusRasterOverflow);
   const unsigned long long tag = ((unsigned long long)nd.slot << 48) | ((unsigned long long)k << 32);
   const uint32_t bin = t / nd.bin_steps - bin0;
@@ -403,169 +173,11 @@ __device__ __forceinline__ void record_warp(const NetDev &nd, const uint32_t (&m
         bulk_prefetch_l2(row + (size_t)nd.M_pad * 4u, pre_w);
         if (gbase + pos < nd.rec_cap) nd.rec_entries[gbase + pos] = tag | id;
         hist[hbase + pos] = id;
-        if (smem_list) smem_list[sbase + pos] = id;
         const uint32_t m = id / (uint32_t)kK;
         red_add_u32(nd.rates + ((size_t)bin * nd.G + m) * 3u + pop_of_local(id - m * (uint32_t)kK), 1u);
         ++pos;
       }
     }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Delay-major delivery (Sec. 2.1.1).  A delivery pass follows the update of
-// every step t with (t + 1) % kmin == 0 (kmin = the smallest delay: the spikes
-// of kmin consecutive steps are delivered together, the paper's exchange step
-// equal to the minimum delay).  It produces the inputs of the next kmin steps
-// T = t + 1 .. t + kmin: for each T, the delay-d group (kmin <= d <= n_delay)
-// of every spike of step T - d, one segment per (spike, d).  Segments are
-// spread over all warps of the grid, `lanes` lanes per segment, and their
-// records are reduced straight into the input buffer of T.
-// ---------------------------------------------------------------------------
-// Slot of step T - d, Tm = T mod D, 1 <= d < D.
-__device__ __forceinline__ uint32_t slot_back(uint32_t Tm, uint32_t d, uint32_t D) { return Tm >= d ? Tm - d : Tm + D - d; }
-
-// Segment prefix of one target step, held in registers across the warp:
-// lane l of chunk c stands for delay d = 32 c + l + 1, with incl[c] = the
-// spikes of steps T - d' summed over kmin <= d' <= d (0 below kmin; past
-// n_delay it stays at the total) and base[c] = the sum below the chunk.
-// NCH = chunks of 32 delays (n_delay <= 32 NCH).  No shared memory.
-template <int NCH>
-struct WarpPrefix {
-  uint32_t incl[NCH];
-  uint32_t base[NCH];
-  uint32_t total;
-};
-
-// T = t + 1 + j with Tm = T mod D; the spikes of step t itself are left out
-// when skip_current.  The count loads of all chunks are issued first.
-template <int NCH>
-__device__ __forceinline__ void warp_prefix(const NetDev &nd, WarpPrefix<NCH> &P, uint32_t Tm, uint32_t j,
-                                            bool skip_current) {
-  const uint32_t lane = lane_id();
-  const uint32_t D = nd.D, dmax = nd.n_delay, kmin = nd.kmin;
-  uint32_t v[NCH];
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) {
-    const uint32_t d = 32u * c + lane + 1u;
-    const bool use = d >= kmin && d <= dmax && !(skip_current && d == j + 1u);
-    v[c] = use ? ld_cg_u32(nd.cnt + slot_back(Tm, d, D)) : 0u;
-  }
-  uint32_t run = 0;
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) {
-    uint32_t x = v[c];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= (uint32_t)o) x += y;
-    }
-    P.base[c] = run;
-    P.incl[c] = x + run;
-    run = __shfl_sync(0xFFFFFFFFu, P.incl[c], 31);
-  }
-  P.total = run;
-}
-
-// The delay d of segment g of this lane's group (smallest d with prefix > g)
-// and the prefix below it; d = 0 when g >= the total.  Called by whole warps:
-// every group's g is tested against a chunk with one ballot.
-template <int NCH>
-__device__ __forceinline__ void find_delay(const WarpPrefix<NCH> &P, uint32_t g, uint32_t lanes, uint32_t &d,
-                                           uint32_t &below) {
-  const uint32_t lane = lane_id(), grp = lane / lanes, gpw = 32u / lanes;
-  d = 0;
-  below = 0;
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) {
-    uint32_t first = 32u;   // this group's first lane of the chunk with prefix > g
-    for (uint32_t q = 0; q < gpw; ++q) {
-      const uint32_t gq = __shfl_sync(0xFFFFFFFFu, g, q * lanes);
-      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, P.incl[c] > gq);
-      if (grp == q && bal) first = (uint32_t)(__ffs(bal) - 1);
-    }
-    const uint32_t prev = __shfl_sync(0xFFFFFFFFu, P.incl[c], (first - 1u) & 31u);
-    if (d == 0 && first < 32u) {
-      d = 32u * c + first + 1u;
-      below = first ? prev : P.base[c];
-    }
-  }
-}
-
-// Prefetch into L2 the next delay group (after record b) of source s's row.
-__device__ __forceinline__ void prefetch_next_group(const NetDev &nd, uint32_t s, const uint16_t *o, uint32_t d,
-                                                    uint32_t b) {
-  if (d >= nd.n_delay) return;
-  const uint32_t c2 = o[d + 1u];
-  if (c2 <= b) return;
-  const uint32_t wb = nd.fmt ? 2u : 4u;
-  const uint8_t *row = nd.rows + (size_t)s * nd.row_bytes;
-  prefetch_range_l2(row + (size_t)b * 4u, (c2 - b) * 4u);
-  prefetch_range_l2(row + (size_t)nd.M_pad * 4u + (size_t)b * wb, (c2 - b) * wb);
-}
-
-// Reduce the records [a, b) of source s's row into `acc_T`, `lanes` lanes
-// (this lane is `sub`), the loads of four records per lane issued first.
-__device__ __forceinline__ void add_records(const NetDev &nd, int32_t *acc_T, uint32_t s, uint32_t a, uint32_t b,
-                                            uint32_t sub, uint32_t lanes) {
-  const uint8_t *row = nd.rows + (size_t)s * nd.row_bytes;
-  const uint32_t *keys = reinterpret_cast<const uint32_t *>(row);
-  const uint8_t *wrow = row + (size_t)nd.M_pad * 4u;
-  for (uint32_t r = a + sub; r < b; r += 4u * lanes) {
-    uint32_t kk[4];
-    int32_t vv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t rr = r + (uint32_t)u * lanes;
-      kk[u] = 0u;
-      vv[u] = 0;
-      if (rr < b) {
-        kk[u] = ld_rec_u32(keys + rr);
-        vv[u] = nd.fmt ? ld_rec_s16(reinterpret_cast<const int16_t *>(wrow) + rr) * 64
-                       : __float2int_rn(__fmul_rn(ld_rec_f32(reinterpret_cast<const float *>(wrow) + rr), 65536.0f));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (r + (uint32_t)u * lanes < b) red_add_s32(acc_T + (kk[u] & 0xFFFFFFu), vv[u]);
-  }
-}
-
-// Segments of the target step with slot Tm (prefix P): the warp takes
-// segments wbase .. wbase + 32 / lanes - 1, then the same plus stride, ...,
-// one per group of `lanes` lanes (this lane is `sub` of group grp).
-template <int NCH>
-__device__ __forceinline__ void deliver_segments(const NetDev &nd, const WarpPrefix<NCH> &P, uint32_t Tm,
-                                                 int32_t *acc_T, uint32_t wbase, uint32_t stride, uint32_t lanes) {
-  const uint32_t D = nd.D;
-  const uint32_t lane = lane_id(), grp = lane / lanes, sub = lane % lanes;
-  for (uint32_t gb = wbase; gb < P.total; gb += stride) {   // warp-uniform
-    const uint32_t g = gb + grp;
-    uint32_t d, below;
-    find_delay<NCH>(P, g, lanes, d, below);
-    if (d == 0) continue;   // g past the total (last round)
-    const uint32_t s = ld_cg_u32(nd.hist + (size_t)slot_back(Tm, d, D) * nd.N_pad + (g - below));
-    const uint16_t *o = nd.offs + (size_t)s * nd.os;
-    add_records(nd, acc_T, s, o[d - 1u], o[d], sub, lanes);
-  }
-}
-
-// Fused step, delivery pass after step t: the delay-kmin records of the
-// block's own spikes of step t, reduced into the input of step t + kmin (the
-// step's spike list is not complete while other blocks still update).
-__device__ void deliver_own(const NetDev &nd, const uint32_t *ids, uint32_t cnt, uint32_t t, uint32_t lanes) {
-  const uint32_t tid = threadIdx.x;
-  const uint32_t grp = tid / lanes, sub = tid % lanes, ngrp = blockDim.x / lanes;
-  const uint32_t kmin = nd.kmin;
-  uint32_t b = t % nd.nbuf + kmin;
-  b = b >= nd.nbuf ? b - nd.nbuf : b;
-  int32_t *acc_T = nd.acc + (size_t)b * nd.N_pad;
-  for (uint32_t j = grp; j < cnt; j += ngrp) {
-    const uint32_t s = ids[j];
-    const uint16_t *o = nd.offs + (size_t)s * nd.os;
-    const uint32_t a = o[kmin - 1u], b = o[kmin];
-    if (sub == 0) prefetch_next_group(nd, s, o, kmin, b);
-    add_records(nd, acc_T, s, a, b, sub, lanes);
   }
 }
 
@@ -862,13 +474,13 @@ __global__ void __launch_bounds__(BLOCK, G == 1 ? 1280 / BLOCK : 1) k_update(con
     if (live[g]) mask[g] = integrate4(nd, n0[g], buf, st4[g], I[g]);
   // record per group whose tile is live (warp-uniform)
   if (live[G - 1]) {
-    record_warp<G>(nd, mask, n0, n_ext, t, slot, k, w.bin0, nullptr, nullptr);
+    record_warp<G>(nd, mask, n0, n_ext, t, slot, k, w.bin0);
   } else {
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       if (live[g]) {
         const uint32_t m1[1] = {mask[g]}, a1[1] = {n0[g]}, e1[1] = {n_ext[g]};
-        record_warp<1>(nd, m1, a1, e1, t, slot, k, w.bin0, nullptr, nullptr);
+        record_warp<1>(nd, m1, a1, e1, t, slot, k, w.bin0);
       }
     }
   }
@@ -930,83 +542,6 @@ __global__ void __launch_bounds__(512, NCH == 1 ? 3 : 2) k_deliver(const __grid_
 }
 
 // ---------------------------------------------------------------------------
-// Kernel: fused step over a table of networks.  A block takes work items
-// (network, 4*blockDim neurons): update and recording with a block-local spike
-// list and, after the last step of an exchange period, the delay-kmin records
-// of those spikes and the item's share of the rest of the network's pass.
-// Update reads input buffer t % nbuf and delivery writes the buffers of steps
-// t + 1 .. t + kmin (nbuf = 2 kmin > kmin: never the one being read), so
-// blocks need no grid-wide barrier; many small blocks per SM let one block's
-// update overlap another's delivery.  Launched with programmatic dependent
-// launch: the prologue (descriptor copy, window read) runs while the previous
-// step drains.
-// ---------------------------------------------------------------------------
-template <int NCH>
-__global__ void __launch_bounds__(512) k_fused(const __grid_constant__ FusedTable tab, uint32_t k) {
-  extern __shared__ __align__(128) uint8_t smem[];   // the item's spike ids (4 * blockDim)
-  __shared__ NetDev nd;
-  __shared__ NetWin s_win;
-  __shared__ uint32_t s_count;
-  __shared__ uint32_t s_net;
-  uint32_t *s_ids = reinterpret_cast<uint32_t *>(smem);
-  const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-  if (threadIdx.x == 0) s_net = 0xFFFFFFFFu;
-  bool waited = false;
-  const uint32_t n_items = *tab.n_items;
-  for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-    const FusedItem item = tab.items[it];
-    __syncthreads();   // the previous item is done with shared memory
-    if (s_net != item.net) {
-      const uint32_t *src = reinterpret_cast<const uint32_t *>(tab.nets + item.net);
-      uint32_t *dst = reinterpret_cast<uint32_t *>(&nd);
-      for (uint32_t i = threadIdx.x; i < sizeof(NetDev) / 4; i += blockDim.x) dst[i] = src[i];
-      if (threadIdx.x == 0) s_win = *reinterpret_cast<const NetWin *>(tab.nets[item.net].win);
-    }
-    if (threadIdx.x == 0) s_count = 0u;
-    __syncthreads();
-    if (threadIdx.x == 0) s_net = item.net;
-    const uint32_t t = s_win.t0 + k;
-    if (t >= s_win.t_end) continue;
-    if (!waited) {     // everything below reads what the previous step wrote
-      pdl_wait();
-      pdl_trigger();
-      waited = true;
-    }
-    const uint32_t n0 = item.n_begin + threadIdx.x * 4u;
-    const uint32_t warp_first = item.n_begin + warp * 128u;
-    const uint32_t tm = t % nd.D, tb = t % nd.nbuf;
-    if (warp_first < nd.N_pad) {
-      uint32_t n_ext[1] = {0};
-      const uint32_t mask[1] = {update4(nd, n0, t, tb, n_ext[0])};
-      const uint32_t a1[1] = {n0};
-      record_warp<1>(nd, mask, a1, n_ext, t, tm, k, s_win.bin0, s_ids, &s_count);
-    }
-    __syncthreads();
-    if ((t + 1u) % nd.kmin == 0u) {   // the last step of an exchange period: delivery pass
-      const uint32_t lanes = tab.lanes;
-      deliver_own(nd, s_ids, s_count, t, lanes);
-      // the item's share of the pass: its network's segments are dealt over
-      // all groups of all the network's items
-      const uint32_t gpb = blockDim.x / lanes, gpw = 32u / lanes;
-      const uint32_t wbase = item.index * gpb + warp * gpw, stride = item.count * gpb;
-      for (uint32_t j = 0; j < nd.kmin; ++j) {
-        uint32_t Tm;
-        int32_t *acc_T;
-        target_of(nd, tm, tb, j, Tm, acc_T);
-        WarpPrefix<NCH> P;
-        warp_prefix<NCH>(nd, P, Tm, j, true);
-        deliver_segments<NCH>(nd, P, Tm, acc_T, wbase, stride, lanes);
-      }
-      if (item.index == 0) clear_next_counts(nd, t);
-    }
-  }
-  if (!waited) {
-    pdl_wait();
-    pdl_trigger();
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
 int device_sm_count() {
@@ -1017,7 +552,6 @@ int device_sm_count() {
 }
 
 static bool valid_lanes(uint32_t lanes) { return lanes == 4 || lanes == 8 || lanes == 16 || lanes == 32; }
-static size_t fused_smem_bytes(int block) { return (size_t)block * 16u; }
 
 // Dynamic shared memory of one construction block: the device's opt-in
 // maximum per block (227 KB on sm_103), never above 227 KB.
@@ -1113,33 +647,6 @@ cudaError_t launch_deliver(const NetDev &nd, uint32_t k, StepMod km, uint32_t la
     return launch_ex(k_deliver<kMaxPreChunks>, dim3((unsigned)blocks), dim3(warps * 32), 0, l2, pdl, s, nd, k, km,
                      lanes);
   return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_fused(const FusedTable &tab, uint32_t k, int block, int blocks, cudaStream_t s) {
-  if (block < 128 || block > 512 || (block % 32) || !valid_lanes(tab.lanes)) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = fused_smem_bytes(block);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (tab.chunks == 1u) return cudaLaunchKernelEx(&cfg, k_fused<1>, tab, k);
-  if (tab.chunks == kMaxPreChunks) return cudaLaunchKernelEx(&cfg, k_fused<kMaxPreChunks>, tab, k);
-  return cudaErrorInvalidValue;
-}
-
-int fused_blocks_per_sm(int block, uint32_t chunks) {
-  int n = 0;
-  cudaError_t e = chunks == 1u
-                      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<1>, block, fused_smem_bytes(block))
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<kMaxPreChunks>, block,
-                                                                      fused_smem_bytes(block));
-  if (e != cudaSuccess) return 1;
-  return n > 0 ? n : 1;
 }
 
 }  // namespace snn

@@ -3,8 +3,7 @@
 Requests (parameters, seed, number of steps, arrival time) are admitted in
 arrival order while the device-memory ledger has room for their footprint;
 admitted networks stay resident on the GPU and every active network advances
-together, one fused kernel per time step for the whole set (``run_batch``), in
-chunks of at most ``chunk_steps``.  Requests that arrive while others run join
+together in lockstep (``run_batch``), in chunks of at most ``chunk_steps``.  Requests that arrive while others run join
 at the next chunk boundary; finished networks leave, their spikes and rate
 counts are read into host memory and their device memory is released.
 
