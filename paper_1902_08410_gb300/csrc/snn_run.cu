@@ -216,15 +216,14 @@ __device__ __forceinline__ uint32_t deliver_front(const NetDev &nd, uint32_t s, 
     uint32_t k[U];
     int32_t v[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) k[u] = i0 + 32u * u < M ? ld_rec_u32(kp + 32 * u) : 0xFFFFFFFFu;
+    for (int u = 0; u < U; ++u) k[u] = ld_rec_u32_if(i0 + 32u * u < M, kp + 32 * u, 0xFFFFFFFFu);
     if (i16) {
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        v[u] = i0 + 32u * u < M ? ld_rec_s16(reinterpret_cast<const int16_t *>(wp) + 32 * u) * 64 : 0;
+      for (int u = 0; u < U; ++u) v[u] = ld_rec_s16_if(i0 + 32u * u < M, reinterpret_cast<const int16_t *>(wp) + 32 * u);
     } else {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        v[u] = i0 + 32u * u < M ? (int32_t)ld_rec_u32(reinterpret_cast<const uint32_t *>(wp) + 32 * u) : 0;
+        v[u] = (int32_t)ld_rec_u32_if(i0 + 32u * u < M, reinterpret_cast<const uint32_t *>(wp) + 32 * u, 0u);
     }
     uint32_t n = 0;
 #pragma unroll
@@ -237,7 +236,7 @@ __device__ __forceinline__ uint32_t deliver_front(const NetDev &nd, uint32_t s, 
         if (b >= to.n) b -= to.n;
         b = buffer_at(b, to.flip, to.gap);
         red_add_s32(acc + (size_t)(b * N_pad + (k[u] & 0xFFFFFFu)),
-                    i16 ? v[u] : __float2int_rn(__fmul_rn(__int_as_float(v[u]), 65536.0f)));
+                    i16 ? v[u] * 64 : __float2int_rn(__fmul_rn(__int_as_float(v[u]), 65536.0f)));
       }
     }
     p += n;
