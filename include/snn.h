@@ -111,7 +111,7 @@ typedef struct snn_launch {
                               fields are at their defaults; 1 = persistent kernel where it fits */
   int32_t update_block;    /* threads per update block: 64 (update_groups 1 only), 128, 256 or 512 */
   int32_t deliver_warps;   /* warps per delivery block: 1..16 */
-  int32_t fused_block;     /* path 1: threads per SM = fused_block * fused_items_per_sm, at most 1024; */
+  int32_t fused_block;     /* path 1: threads per SM = fused_block * fused_items_per_sm, at most 640; */
   int32_t fused_items_per_sm; /* fused_block 128..512, fused_items_per_sm 1..32 */
   int32_t window_steps;    /* steps per window: one launch or captured CUDA graph (1..4096) */
   int32_t deliver_lanes;   /* lanes that share one (spike, delay) segment of records: 4, 8, 16, 32 */

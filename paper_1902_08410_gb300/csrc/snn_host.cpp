@@ -1530,7 +1530,7 @@ extern "C" int snn_autotune_batch(const snn_handle *hs, int32_t n, uint32_t tria
   float orig_ms = 1e30f, best_ms = 1e30f;
   snn_launch best = orig;
   int status = trial(orig, 2, &orig_ms);
-  for (int ips : {2, 4, 6, 8}) {   // 256 .. 1024 threads per SM
+  for (int ips : {2, 3, 4, 5}) {   // 256 .. 640 threads per SM
     if (status != SNN_OK) break;
     snn_launch c = orig;
     c.fused_block = 128;
@@ -1715,7 +1715,7 @@ static int autotune_impl(snn_net *h, uint32_t trial_steps, int path_only) {
       c.update_groups = ug;
       cands.push_back(c);
     }
-  for (int ips : {4, 8}) {
+  for (int ips : {3, 5}) {
     if (path_only == 0) continue;
     snn_launch c = orig;
     c.path = 1;

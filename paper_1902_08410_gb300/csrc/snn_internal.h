@@ -153,6 +153,7 @@ struct RunArgs {
   uint32_t visit;             // steps between two visits of a live spike (1 in the period form)
   uint32_t fifo;              // live spikes of one ring that a block holds in shared memory (power of two)
   uint32_t nt;                // tiles of a block, at most
+  uint32_t drives;            // external drives kept per neuron: kmin in the period form, else 1 or 2
   uint32_t pre;               // records of a new spike's row prefetched (multiple of 8)
   // {grid barrier count, last step (+1) that overflowed a live list, lists not taken over}, zero at launch
   uint32_t *bar;
@@ -161,7 +162,7 @@ struct RunArgs {
 struct RunShape {
   int blocks = 0, threads = 0;
   int form = 0;               // RunForm
-  uint32_t fifo = 0, nt = 0, visit = 1;
+  uint32_t fifo = 0, nt = 0, visit = 1, drives = 1;
   size_t smem = 0;
 };
 // blocks == 0: too many tiles for one launch.

@@ -42,7 +42,7 @@
 
 namespace snn {
 
-constexpr int kRunThreads = 1024;
+constexpr int kRunThreads = 640;
 constexpr uint32_t kPendCap = 1024;      // neurons with two or more external events listed per step and block
 constexpr uint32_t kSpinLimit = 1u << 22;   // barrier polls (about a microsecond each) before giving up
 
@@ -59,6 +59,12 @@ __device__ __forceinline__ void live_unpack(unsigned long long e, uint32_t &id, 
   net = hi >> 16;
 }
 
+// Neurons of one step's drive with more than one external event: index in the drives << 5 | events.
+struct Pending {
+  uint32_t n;
+  uint32_t list[kPendCap];
+};
+
 struct RunShared {
   NetDev nd;                          // single network
   // Live spikes by (step of the spike mod visit): ring c holds those visited after the steps k = c mod visit.
@@ -66,7 +72,7 @@ struct RunShared {
   uint32_t base[kMaxVisit];           // the same before this step
   uint32_t head[kMaxVisit];           // first entry that may still be alive
   struct {
-    uint32_t next, draw, npend;       // next live spike, (tile, step) unit, listed neuron
+    uint32_t next, draw;              // next live spike, (tile, step) unit
   } ctr[2];                           // of this interval and, cleared ahead, the next
   uint32_t abort;
   uint32_t end_k;                     // next step of the window at which a network has stopped before the others
@@ -74,7 +80,7 @@ struct RunShared {
   int lo_list;                        // first step (of the window) the global lists are read from
   unsigned long long live0;
   uint32_t tail_at[512];              // tail of the ring of step k after it, at k mod 512 (above n_delay + visit)
-  uint32_t pend[kPendCap];
+  Pending pend[2];
 };
 
 template <bool MULTI>
@@ -181,9 +187,10 @@ enum RunForm { kAhead, kPeriod };
 // acc[t0 mod 2] and acc[(t0 + 1) mod 2] (flip = t0 mod 2); the rest lie behind
 // the D spike lists that follow acc.  kPeriod: buffer t mod nbuf (flip = gap = 0).
 __device__ __forceinline__ uint32_t buffer_at(uint32_t r, uint32_t flip, uint32_t gap) { return r < 2u ? r ^ flip : r + gap; }
+// kAhead: r = k mod (visit + 2), k a step of the window that starts at t0.
 template <int FORM>
-__device__ __forceinline__ int32_t *input_of(const RunArgs &a, const NetDev &nd, uint32_t t0, uint32_t k) {
-  const uint32_t b = FORM == kAhead ? buffer_at(k % (a.visit + 2u), t0 & 1u, nd.D) : (t0 + k) % nd.nbuf;
+__device__ __forceinline__ int32_t *input_of(const NetDev &nd, uint32_t t0, uint32_t k, uint32_t r) {
+  const uint32_t b = FORM == kAhead ? buffer_at(r, t0 & 1u, nd.D) : (t0 + k) % nd.nbuf;
   return nd.acc + (size_t)b * nd.N_pad;
 }
 
@@ -195,8 +202,8 @@ struct Due {
 };
 // Records due after step k (relative to a window that starts at t0) of a spike `age` steps old.
 template <int FORM>
-__device__ __forceinline__ Due due_at(const RunArgs &a, const NetDev &nd, uint32_t t0, uint32_t k, int age) {
-  if constexpr (FORM == kAhead) return Due{(int)(k % (a.visit + 2u)) - age, a.visit + 2u, t0 & 1u, nd.D};
+__device__ __forceinline__ Due due_at(const RunArgs &a, const NetDev &nd, uint32_t t0, uint32_t k, uint32_t r, int age) {
+  if constexpr (FORM == kAhead) return Due{(int)r - age, a.visit + 2u, t0 & 1u, nd.D};
   else return Due{(int)((t0 + k) % nd.nbuf) - age, nd.nbuf, 0u, 0u};
 }
 
@@ -360,7 +367,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   __shared__ RunShared s;
   constexpr bool PERIOD = FORM == kPeriod;
   const uint32_t nt = blockIdx.x < a.n_tiles ? (a.n_tiles - 1u - blockIdx.x) / gridDim.x + 1u : 0u;
-  const uint32_t P = PERIOD ? a.kmin : 1u;     // drives kept per tile
+  const bool deep = !PERIOD && a.drives == 2u;   // drives are drawn two steps ahead
+  const uint32_t P = a.drives;                   // drives kept per tile
   const uint32_t C = PERIOD ? 1u : a.visit, cap = a.fifo;
   // live spikes of ring c at c * cap
   unsigned long long *live = reinterpret_cast<unsigned long long *>(smem);
@@ -381,7 +389,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   }
   if (tid == 0) {
     for (uint32_t c = 0; c < kMaxVisit; ++c) s.tail[c] = s.base[c] = s.head[c] = 0u;
-    for (uint32_t i = 0; i < 2u; ++i) s.ctr[i].next = s.ctr[i].draw = s.ctr[i].npend = 0u;
+    for (uint32_t i = 0; i < 2u; ++i) s.ctr[i].next = s.ctr[i].draw = s.pend[i].n = 0u;
     s.abort = 0u;
     s.live0 = 0ull;
     s.last_list = -100000;
@@ -481,7 +489,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
 
   // The records of live entry e of ring c for the steps of the window up to
   // `upto`, after step k.  Whole warp, 32 U records in flight.
-  auto visit = [&](auto U, uint32_t c, uint32_t e, uint32_t k, uint32_t upto) {
+  auto visit = [&](auto U, uint32_t c, uint32_t e, uint32_t k, uint32_t r, uint32_t upto) {
     unsigned long long *at = live + c * cap + (e & (cap - 1u));
     uint32_t id, p, net;
     int kts;
@@ -493,24 +501,24 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     const int dlim = (int)(PERIOD ? upto : min(upto, adv)) - kts;
     if (PERIOD ? k >= adv : dlim <= 0) return;
     const uint32_t q = deliver_front<decltype(U)::n>(nd, id, p, (uint32_t)min(dlim, 254),
-                                                     due_at<FORM>(a, nd, w.t0, k, (int)k - kts));
+                                                     due_at<FORM>(a, nd, w.t0, k, r, (int)k - kts));
     if (q != p && lane == 0) *at = live_pack(id, kts, q, net);
   };
 
   // The entries [from, to) of ring c as they come, their records for steps up to `upto`, after step k.
-  auto visit_all = [&](uint32_t c, uint32_t from, uint32_t to, uint32_t k, uint32_t upto, uint32_t ci) {
+  auto visit_all = [&](uint32_t c, uint32_t from, uint32_t to, uint32_t k, uint32_t r, uint32_t upto, uint32_t ci) {
     while (true) {
       uint32_t e = 0;
       if (lane == 0) e = atomicAdd(&s.ctr[ci].next, 1u);
       e = from + __shfl_sync(0xFFFFFFFFu, e, 0);
       if (e >= to) break;
-      visit(Width<8>{}, c, e, k, upto);
+      visit(Width<8>{}, c, e, k, r, upto);
     }
   };
 
   // External drive of the block's tiles at steps k .. k + L - 1 into s_I: (tile,
   // step) units taken as they come
-  auto draw = [&](uint32_t k, uint32_t L, uint32_t ci) {
+  auto draw = [&](uint32_t k, uint32_t L, uint32_t ci, Pending &pend) {
     const uint32_t units = nt * L;
     while (true) {
       uint32_t u = 0;
@@ -523,7 +531,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
       const NetWin w = win_of<MULTI>(a, tile.x);
       const uint32_t t = w.t0 + k + i;
       if (t >= w.t_end) continue;
-      const uint32_t n0 = tile.y + lane * 4u, slot = j * P + i;
+      const uint32_t n0 = tile.y + lane * 4u, slot = PERIOD ? j * P + i : (deep ? j * 2u + (k & 1u) : j);
       int p0, p1;
       pair_pops(n0, p0, p1);
       uint32_t kx[4];
@@ -540,20 +548,20 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         if (kx[q] > 1u) {
-          const uint32_t at = atomicAdd(&s.ctr[ci].npend, 1u), n = slot * 128u + lane * 4u + q;
+          const uint32_t at = atomicAdd(&pend.n, 1u), n = slot * 128u + lane * 4u + q;
           if (at < kPendCap)
-            s.pend[at] = (n << 5) | kx[q];
+            pend.list[at] = (n << 5) | kx[q];
           else
             reinterpret_cast<int32_t *>(s_I)[n] += extra_sum(nd, q < 2 ? p0 : p1, kx[q], n0 + q, t);
         }
     }
   };
   // events after the first of the listed neurons, one neuron per thread (the last warps first)
-  auto draw_more = [&](uint32_t k, uint32_t ci) {
-    const uint32_t np = min(s.ctr[ci].npend, kPendCap);
+  auto draw_more = [&](uint32_t k, const Pending &pend) {
+    const uint32_t np = min(pend.n, kPendCap);
     for (uint32_t x = (nw - 1u - warp) * 32u + lane; x < np; x += blockDim.x) {
-      const uint32_t e = s.pend[x], at = e >> 5, kx = e & 31u;
-      const uint32_t slot = at >> 7, j = PERIOD ? slot / P : slot, i = slot - j * P;
+      const uint32_t e = pend.list[x], at = e >> 5, kx = e & 31u;
+      const uint32_t slot = at >> 7, j = PERIOD ? slot / P : slot >> (deep ? 1 : 0), i = PERIOD ? slot - j * P : 0u;
       const uint2 tile = s_tile[j];
       const NetDev &nd = net_of<MULTI>(a, s, tile.x);
       const uint32_t n = tile.y + (at & 127u);
@@ -566,18 +574,26 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     return PERIOD ? min(a.kmin - (phase0 + k) % a.kmin, a.steps - k) : 1u;
   };
   __syncthreads();
-  draw(0u, interval(0u), (met & 1u) ^ 1u);
+  draw(0u, interval(0u), (met & 1u) ^ 1u, s.pend[0]);
   if constexpr (!PERIOD) {   // up to the steps that the first visit of each ring leaves out
     for (uint32_t c = 0; c < C; ++c)
-      for (uint32_t e = warp; e < s.base[c]; e += nw) visit(Width<8>{}, c, e, 0u, c + 1u);
+      for (uint32_t e = warp; e < s.base[c]; e += nw) visit(Width<8>{}, c, e, 0u, 0u, c + 1u);
   }
   __syncthreads();
-  draw_more(0u, (met & 1u) ^ 1u);
+  draw_more(0u, s.pend[0]);
+  if (deep) {
+    if (tid == 0) s.ctr[(met & 1u) ^ 1u].draw = 0u;
+    __syncthreads();
+    if (1u < a.steps) draw(1u, 1u, (met & 1u) ^ 1u, s.pend[1]);
+  }
+  __syncthreads();
+  if (tid == 0) s.pend[0].n = 0u;
   __syncthreads();
 
+  uint32_t rk = 0, ck = 0;   // k mod (visit + 2), k mod visit
   for (uint32_t k = 0; k < a.steps && !s.abort;) {
     const uint32_t L = interval(k), kl = k + L - 1u;   // steps of this interval, its last step
-    const uint32_t ring = PERIOD ? 0u : k % C, ci = met & 1u;
+    const uint32_t ring = PERIOD ? 0u : ck, ci = met & 1u;
     const uint32_t base = s.base[ring], head = s.head[ring];
     unsigned long long *rlive = live + ring * cap;
     if constexpr (MULTI) {
@@ -610,8 +626,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
       auto load = [&](uint32_t i0) {
 #pragma unroll
         for (uint32_t i = 0; i < IN; ++i)
-          I[i] = i0 + i < Ln ? ld_cg_i4(reinterpret_cast<const int4 *>(input_of<FORM>(a, nd, w.t0, k + i0 + i)) + i4)
-                            : make_int4(0, 0, 0, 0);
+          I[i] = i0 + i < Ln ? ld_cg_i4(reinterpret_cast<const int4 *>(input_of<FORM>(nd, w.t0, k + i0 + i, rk)) + i4)
+                             : make_int4(0, 0, 0, 0);
       };
       load(0u);
       int p0, p1;
@@ -624,9 +640,9 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
         for (uint32_t i = 0; i < IN; ++i) {
           if (i0 + i >= Ln) break;
           const uint32_t ki = k + i0 + i;
-          int4 E = s_I[(j * P + i0 + i) * 32u + lane];
+          int4 E = s_I[(PERIOD ? j * P + i0 + i : (deep ? j * 2u + (k & 1u) : j)) * 32u + lane];
           if (I[i].x | I[i].y | I[i].z | I[i].w) {
-            reinterpret_cast<int4 *>(input_of<FORM>(a, nd, w.t0, ki))[i4] = make_int4(0, 0, 0, 0);
+            reinterpret_cast<int4 *>(input_of<FORM>(nd, w.t0, ki, rk))[i4] = make_int4(0, 0, 0, 0);
             E.x += I[i].x;
             E.y += I[i].y;
             E.z += I[i].z;
@@ -665,7 +681,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
               // the pass that ends the interval reaches steps up to kl + kmin
               const uint32_t age = kl - ki;
               spill_spikes(a, nd, w, n0, full, ki, w.t0 + kl < w.t_end && pass_after(nd, w.t0 + kl) ? age + nd.kmin : 0u,
-                           due_at<FORM>(a, nd, w.t0, kl, (int)age));
+                           due_at<FORM>(a, nd, w.t0, kl, rk, (int)age));
             }
           }
         }
@@ -690,23 +706,24 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     auto visit_and_draw = [&](bool visits, uint32_t upto) {
       for (uint32_t i = 0; i < 2u; ++i) {
         if ((i ^ warp) & 1u) {
-          if (more) draw(k + L, interval(k + L), ci);
+          const uint32_t kd = deep ? k + 2u : k + L;
+          if (kd < a.steps) draw(kd, interval(kd), ci, s.pend[PERIOD ? ci : kd & 1u]);
         } else {
-          if (visits) visit_all(ring, head, tail, kl, upto, ci);
+          if (visits) visit_all(ring, head, tail, kl, rk, upto, ci);
         }
       }
     };
     if constexpr (PERIOD) {
       visit_and_draw((phase0 + kl + 1u) % a.kmin == 0u, kl + a.kmin);
     } else {
-      for (uint32_t e = base + warp; e < tail; e += nw) visit(Width<3>{}, ring, e, k, k + 1u);
+      for (uint32_t e = base + warp; e < tail; e += nw) visit(Width<3>{}, ring, e, k, rk, k + 1u);
     }
     if (s.last_list >= (int)kl + 1 - (int)a.nd_max) {   // global lists hold live spikes (block-uniform)
       const uint32_t gw = blockIdx.x * nw + warp, total = gridDim.x * nw;
       auto lists = [&](const NetDev &nd, const NetWin &w, uint32_t wi, uint32_t wn) {
         if (w.t0 + kl < w.t_end && pass_after(nd, w.t0 + kl))
           deliver_lists(nd, w.t0 + kl, s.lo_list - (int)kl, (int)k - (int)kl, wi, wn,
-                        PERIOD ? nullptr : input_of<FORM>(a, nd, w.t0, k + 1u));
+                        PERIOD ? nullptr : input_of<FORM>(nd, w.t0, k + 1u, rk + 1u == a.visit + 2u ? 0u : rk + 1u));
       };
       if constexpr (!MULTI) {
         lists(s.nd, a.win, gw, total);
@@ -721,7 +738,10 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
         }
       }
     }
-    if (tid == 0) s.ctr[ci ^ 1u].next = s.ctr[ci ^ 1u].draw = s.ctr[ci ^ 1u].npend = 0u;   // last used before the barrier before
+    if (tid == 0) {   // last used before the barrier before
+      s.ctr[ci ^ 1u].next = s.ctr[ci ^ 1u].draw = 0u;
+      s.pend[PERIOD ? ci ^ 1u : (k + (deep ? 2u : 1u)) & 1u].n = 0u;
+    }
     __syncthreads();
 
     // ---- arrive; record, visit and draw; wait
@@ -752,11 +772,16 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
         if (e < tail) record_at(net_of<MULTI>(a, s, net), win_of<MULTI>(a, net), at, id, (uint32_t)kts);
       }
     }
-    if (!PERIOD && more) {
+    if constexpr (PERIOD) {
+      if (more) draw_more(k + L, s.pend[ci]);
+    } else if (more) {
+      if (deep) draw_more(k + 1u, s.pend[(k + 1u) & 1u]);   // drawn in the last interval
       visit_and_draw(true, k + C + 1u);
-      __syncthreads();
+      if (!deep) {
+        __syncthreads();
+        draw_more(k + 1u, s.pend[(k + 1u) & 1u]);
+      }
     }
-    if (more) draw_more(k + L, ci);
     if (tid == 0) {
       grid_wait(a, s, met);
       const uint32_t over = ld_cg_u32(a.bar + 1);
@@ -764,6 +789,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     }
     __syncthreads();
     k += L;
+    rk = rk + 1u == a.visit + 2u ? 0u : rk + 1u;
+    ck = ck + 1u == C ? 0u : ck + 1u;
   }
 
   // ---- epilogue: live spikes, external events, inputs and state back to global memory
@@ -783,7 +810,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     const uint32_t n0 = tile.y + lane * 4u, i4 = n0 >> 2;
     if (n0 >= nd.N) continue;
     if constexpr (!PERIOD) {   // the input of the next step goes where the other paths read it
-      int4 *from = reinterpret_cast<int4 *>(input_of<FORM>(a, nd, w.t0, w.t_end - w.t0)) + i4;
+      const uint32_t adv = w.t_end - w.t0;
+      int4 *from = reinterpret_cast<int4 *>(input_of<FORM>(nd, w.t0, adv, adv % (a.visit + 2u))) + i4;
       int4 *to = reinterpret_cast<int4 *>(nd.acc + (size_t)(w.t_end & 1u) * nd.N_pad) + i4;
       if (from != to) {
         *to = ld_cg_i4(from);
@@ -800,9 +828,9 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
 // Shape and launch
 // ---------------------------------------------------------------------------
 // Shared memory of a block with nt tiles: live lists, tile table, and per
-// neuron `period` drives (4 bytes each), V, c and the refractory counter.
-static size_t run_smem(uint32_t period, uint32_t nt, uint32_t entries) {
-  return (((size_t)entries * 8u + (size_t)nt * 12u + 15u) & ~(size_t)15u) + (size_t)nt * 128u * (4u * period + 9u);
+// neuron `drives` drives (4 bytes each), V, c and the refractory counter.
+static size_t run_smem(uint32_t drives, uint32_t nt, uint32_t entries) {
+  return (((size_t)entries * 8u + (size_t)nt * 12u + 15u) & ~(size_t)15u) + (size_t)nt * 128u * (4u * drives + 9u);
 }
 
 // Dynamic shared memory of a block: the opt-in maximum less the static part.
@@ -834,9 +862,10 @@ cudaError_t prepare_run_kernels() {
   return cudaSuccess;
 }
 
-// One block per SM, or per tile where there are fewer tiles; 1024 threads (64
-// registers) but fewer for a few tiles, where the block barriers cost more than
-// further warps give.  The form fits as long as the state and `kmin` drives per
+// One block per SM, or per tile where there are fewer tiles; 640 threads (96
+// registers, no spills; 1024: 4-10% more time a step from 4x4 to 40x40 modules,
+// 512: 8% more from 16x16 on) but fewer for a few tiles, where the block barriers
+// cost more than further warps give.  The form fits as long as the state and `kmin` drives per
 // neuron stay in shared memory (2.1M neurons at kmin = 1); what does not fit
 // takes two kernels per step (64x64 modules: 105 us a step, against 125 and 217 us
 // in two forms of this kernel with the state in global memory).
@@ -851,8 +880,11 @@ RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads) {
   sh.visit = sh.form == kAhead ? kMaxVisit : 1u;
   const size_t budget = run_smem_budget();
   sh.fifo = 512u;
-  while (sh.fifo < 8192u / sh.visit && run_smem(kmin, sh.nt, sh.visit * sh.fifo * 2u) <= budget) sh.fifo *= 2u;
-  sh.smem = run_smem(kmin, sh.nt, sh.visit * sh.fifo);
+  // Drives a step further ahead where they fit: the neurons with several external events are then completed beside
+  // the visits instead of behind a block barrier.
+  sh.drives = sh.form == kPeriod ? kmin : (run_smem(2u, sh.nt, sh.visit * sh.fifo) <= budget ? 2u : 1u);
+  while (sh.fifo < 8192u / sh.visit && run_smem(sh.drives, sh.nt, sh.visit * sh.fifo * 2u) <= budget) sh.fifo *= 2u;
+  sh.smem = run_smem(sh.drives, sh.nt, sh.visit * sh.fifo);
   if (sh.smem > budget) sh.blocks = 0;   // too many tiles per block
   return sh;
 }
@@ -864,6 +896,7 @@ cudaError_t launch_run(const RunArgs &args, const RunShape &sh, const L2Window &
   a.fifo = sh.fifo;
   a.nt = sh.nt;
   a.visit = sh.visit;
+  a.drives = sh.drives;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)sh.blocks);
   cfg.blockDim = dim3((unsigned)sh.threads);
