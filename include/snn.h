@@ -117,11 +117,11 @@ typedef struct snn_launch {
   int32_t deliver_lanes;   /* lanes that share one (spike, delay) segment of records: 4, 8, 16, 32 */
   int32_t update_groups;   /* groups of 4 neurons per update thread: 1, 2 or 4
                               (512-thread blocks: 1 or 2) */
-  int32_t l2_persist;      /* two-kernel path: 1 = the neuron state and input buffers are
-                              given a persisting L2 access-policy window (the CUDA
-                              context's persisting set-aside is raised to the device
-                              maximum while any such network lives, then restored);
-                              0 = normal caching */
+  int32_t l2_persist;      /* 1 = the neuron state and input buffers are given a persisting
+                              L2 access-policy window where they fit the device's largest
+                              set-aside together (the CUDA context's persisting set-aside
+                              is raised to that while any such network lives, then
+                              restored); 0 = normal caching */
   int32_t deliver_blocks;  /* delivery blocks per SM: 1..32 (the grid is SMs x deliver_blocks;
                               every warp takes (spike, delay) segments of the pass) */
   int32_t overlap;         /* two-kernel path: 1 = the kernels of consecutive steps overlap

@@ -432,19 +432,23 @@ static void l2_release(snn_net *h) {
   }
 }
 
-// Bytes of the persisting window at the start of the arena: V, c, ref, the
-// input buffers and the spike counts when they fit the set-aside together,
-// else V, c and ref alone.  The spike lists (sparse: only the ids of recent
-// spikes are touched) are never part of it.
+// Bytes of the persisting window at the start of the arena: V, c, ref, the spike
+// counts and the input buffers when they fit the largest set-aside together,
+// else none, and no set-aside is taken from the other lines (us a step at 5.12M neurons:
+// 80; 90-98 with V, c and ref alone in the window, 110-120 with the
+// set-aside raised and no window; 3.92M neurons, which fit: 57 in it, 61 without).
+// The spike lists (sparse: only the ids of recent spikes are touched) are never
+// part of it.
 static size_t l2_window_bytes(const snn_net *h) {
-  int dev = 0, max_win = 0;
+  int dev = 0, max_win = 0, max_persist = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&max_win, cudaDevAttrMaxAccessPolicyWindowSize, dev) != cudaSuccess) {
+      cudaDeviceGetAttribute(&max_win, cudaDevAttrMaxAccessPolicyWindowSize, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&max_persist, cudaDevAttrMaxPersistingL2CacheSize, dev) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  const size_t all = h->L.off_hist, state = h->L.off_cnt;
-  return std::min<size_t>(all <= g_l2_setaside ? all : state, (size_t)max_win);
+  const size_t all = h->L.off_hist;
+  return all <= (size_t)max_persist ? std::min<size_t>(all, (size_t)max_win) : 0;
 }
 
 // The persisting window of network h.  Networks that run at the same time
@@ -454,10 +458,11 @@ static size_t l2_window_bytes(const snn_net *h) {
 static int l2_window(snn_net *h, L2Window *out) {
   *out = L2Window{};
   if (!h->cfg.l2_persist) return SNN_OK;
+  const size_t bytes = l2_window_bytes(h);
+  if (bytes == 0) return SNN_OK;
   int rc = l2_acquire(h);
   if (rc) return rc;
-  const size_t bytes = l2_window_bytes(h);
-  if (bytes == 0 || g_l2_setaside == 0) return SNN_OK;
+  if (g_l2_setaside == 0) return SNN_OK;
   out->base = h->arena.p;
   out->bytes = bytes;
   out->hit_ratio = (float)std::min(1.0, (double)g_l2_setaside / (double)bytes);
@@ -565,14 +570,7 @@ static void fill_descriptor(snn_net *h) {
   d.nbuf = L.nbuf;
   for (int q = 0; q < 3; ++q) {
     const PopTables t = pop_tables(h->p, q);
-    d.pvv[q] = t.pvv;
-    d.pvc[q] = t.pvc;
-    d.pcc[q] = t.pcc;
-    d.el[q] = h->p.E_L[q];
     d.vth[q] = h->p.V_th[q];
-    d.vr[q] = h->p.V_r[q];
-    d.alpha[q] = h->p.alpha_c[q];
-    d.narp[q] = t.narp;
     float narp_bits;
     std::memcpy(&narp_bits, &t.narp, 4);
     d.pa[q] = make_float4(t.pvv, t.pvc, t.pcc, h->p.E_L[q]);

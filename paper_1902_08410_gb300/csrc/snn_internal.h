@@ -73,13 +73,10 @@ struct alignas(16) NetDev {
   uint32_t pad1;
 
   // --- per population constants (Eq. 2 propagators, Table S1)
-  float pvv[kNPop], pvc[kNPop], pcc[kNPop];
-  float el[kNPop], vth[kNPop], vr[kNPop], alpha[kNPop];
-  int32_t narp[kNPop];
-  uint32_t pad0[2];
+  float vth[kNPop];
   alignas(16) uint32_t thr[kNPop][kPoisMax];   // Poisson CDF thresholds, scaled by 2^20 (read four at a time)
-  // the same constants as two 16-byte loads per population: {pvv, pvc, pcc, el}
-  // and {vth, vr, alpha, narp (bits)}
+  // two 16-byte loads per population: {P_VV, P_Vc, P_cc, E} and {V_th, V_r,
+  // alpha, refractory steps (bits)}
   float4 pa[kNPop], pb[kNPop];
 
   // --- device arrays

@@ -57,54 +57,37 @@ __device__ __forceinline__ void load_input4(const NetDev &nd, uint32_t n0, uint3
   g.I = ld_cg_i4(reinterpret_cast<const int4 *>(nd.acc + (size_t)buf * nd.N_pad) + (n0 >> 2));
 }
 
-// External drive of 4 neurons at step t (Poisson counts from one
-// counter-based draw, word n mod 4 each; amplitudes from the table): adds the
-// drive to I and the number of external events of the live neurons to n_ext.
-// Reads only the parameters and the amplitude table.
-__device__ __forceinline__ void drive4(const NetDev &nd, uint32_t n0, uint32_t t, int32_t (&I)[4], uint32_t &n_ext) {
-  const uint4 R = philox4x32_10(n0 >> 2, t, 1u, 0u, nd.key0, nd.key1);
-  const uint32_t Wv[4] = {R.x, R.y, R.z, R.w};
-  uint32_t local = n0 % (uint32_t)kK;
-  int pops[4];
+// External drive of 4 neurons at step t: adds the drive to I and the number of
+// external events of the live neurons to n_ext.  Reads only the parameters and
+// the amplitude table.
+__device__ __forceinline__ void drive4(const NetDev &nd, uint32_t n0, uint32_t t, int p0, int p1, int32_t (&I)[4],
+                                       uint32_t &n_ext) {
   uint32_t kx[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    pops[q] = pop_of_local(local);
-    kx[q] = poisson_count(nd, pops[q], Wv[q]);
-    local = (local + 1u == (uint32_t)kK) ? 0u : local + 1u;
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q)   // first external event: independent table loads
-    if (kx[q]) I[q] += __ldg(nd.amp + pops[q] * kZTab + (Wv[q] & 0xFFFu));
+  const int4 E = first_drive(nd, n0, t, p0, p1, kx);
+  I[0] += E.x;
+  I[1] += E.y;
+  I[2] += E.z;
+  I[3] += E.w;
   extra_events_warp(nd, n0, t, kx, I);
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (n0 + q < nd.N) n_ext += kx[q];
+  if (n0 < nd.N) n_ext += kx[0] + kx[1];
+  if (n0 + 2u < nd.N) n_ext += kx[2] + kx[3];
 }
 
 // Advance the 4 neurons of g by one step (Eq. 2) with total input I (the
 // external drive plus the buffer g.I), store the state and clear input buffer
 // `buf`; returns the 4-bit spike mask.  Integer input: the order in which the
 // drive and the buffer are summed does not change the result.
-__device__ __forceinline__ uint32_t integrate4(const NetDev &nd, uint32_t n0, uint32_t buf, const Group4 &g,
+__device__ __forceinline__ uint32_t integrate4(const NetDev &nd, uint32_t n0, uint32_t buf, int p0, int p1, Group4 &g,
                                                const int32_t (&I)[4]) {
-  const int32_t Iv[4] = {I[0] + g.I.x, I[1] + g.I.y, I[2] + g.I.z, I[3] + g.I.w};
-  float Vv[4] = {g.V.x, g.V.y, g.V.z, g.V.w};
-  float cv[4] = {g.c.x, g.c.y, g.c.z, g.c.w};
-  uint32_t rv[4] = {g.ref & 0xFFu, (g.ref >> 8) & 0xFFu, (g.ref >> 16) & 0xFFu, g.ref >> 24};
-  uint32_t mask = 0;
-  uint32_t local = n0 % (uint32_t)kK;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (n0 + q < nd.N && neuron_step(nd, pop_of_local(local), Vv[q], cv[q], rv[q], Iv[q])) mask |= 1u << q;
-    local = (local + 1u == (uint32_t)kK) ? 0u : local + 1u;
-  }
+  const uint32_t mask =
+      run_step4(nd, n0, p0, p1, g.V, g.c, g.ref, make_int4(I[0] + g.I.x, I[1] + g.I.y, I[2] + g.I.z, I[3] + g.I.w));
   if (n0 < nd.N) {
     const uint32_t i4 = n0 >> 2;
-    reinterpret_cast<float4 *>(nd.V)[i4] = make_float4(Vv[0], Vv[1], Vv[2], Vv[3]);
-    reinterpret_cast<float4 *>(nd.c)[i4] = make_float4(cv[0], cv[1], cv[2], cv[3]);
-    reinterpret_cast<uint32_t *>(nd.ref)[i4] = rv[0] | (rv[1] << 8) | (rv[2] << 16) | (rv[3] << 24);
-    reinterpret_cast<int4 *>(nd.acc + (size_t)buf * nd.N_pad)[i4] = make_int4(0, 0, 0, 0);
+    reinterpret_cast<float4 *>(nd.V)[i4] = g.V;
+    reinterpret_cast<float4 *>(nd.c)[i4] = g.c;
+    reinterpret_cast<uint32_t *>(nd.ref)[i4] = g.ref;
+    if (g.I.x | g.I.y | g.I.z | g.I.w)
+      reinterpret_cast<int4 *>(nd.acc + (size_t)buf * nd.N_pad)[i4] = make_int4(0, 0, 0, 0);
   }
   return mask;
 }
@@ -460,7 +443,12 @@ __global__ void __launch_bounds__(kBuildWarpsMax * 32) k_build_rows(const __grid
 // that follows the wait lets the delivery pass after this step start on older
 // spikes.
 // One group per thread is capped at 48 registers (40 resident warps per SM), so
-// that a 720k-neuron grid (37 warps per SM) runs in a single wave.
+// that a 720k-neuron grid (37 warps per SM) runs in a single wave; at 5.12M
+// neurons 64 registers and 32 warps take the same 34.6 us, 40 registers and 48
+// warps 40.7.  There the state and inputs (133 MB a step, about the size of L2)
+// bound it; the branchless step with two parameter loads per pair of neurons
+// brought it from 39.2 us (a loop over the thresholds and seven parameter loads
+// per neuron).
 template <int BLOCK, int G>
 __global__ void __launch_bounds__(BLOCK, G == 1 ? 1280 / BLOCK : 1) k_update(const __grid_constant__ NetDev nd,
                                                                            uint32_t k, StepMod km) {
@@ -486,12 +474,16 @@ __global__ void __launch_bounds__(BLOCK, G == 1 ? 1280 / BLOCK : 1) k_update(con
       if (!km.overlapped) load_input4(nd, n0[g], km.buf, st4[g]);
     }
   int32_t I[G][4];
+  int p0[G], p1[G];
   uint32_t n_ext[G];
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     I[g][0] = I[g][1] = I[g][2] = I[g][3] = 0;
     n_ext[g] = 0;
-    if (live[g]) drive4(nd, n0[g], t, I[g], n_ext[g]);
+    if (live[g]) {
+      pair_pops(n0[g], p0[g], p1[g]);
+      drive4(nd, n0[g], t, p0[g], p1[g], I[g], n_ext[g]);
+    }
   }
   pdl_wait();      // the previous kernel (and everything before it) is complete
   pdl_trigger();
@@ -504,7 +496,7 @@ __global__ void __launch_bounds__(BLOCK, G == 1 ? 1280 / BLOCK : 1) k_update(con
   }
 #pragma unroll
   for (int g = 0; g < G; ++g)
-    if (live[g]) mask[g] = integrate4(nd, n0[g], buf, st4[g], I[g]);
+    if (live[g]) mask[g] = integrate4(nd, n0[g], buf, p0[g], p1[g], st4[g], I[g]);
   // record per group whose tile is live (warp-uniform)
   if (live[G - 1]) {
     record_warp<G>(nd, mask, n0, n_ext, t, slot, k, w.bin0);

@@ -95,77 +95,6 @@ __device__ __forceinline__ NetWin win_of(const RunArgs &a, uint32_t net) {
 }
 __device__ __forceinline__ bool pass_after(const NetDev &nd, uint32_t t) { return nd.kmin == 1u || (t + 1u) % nd.kmin == 0u; }
 
-// Populations of the pairs (n0, n0 + 1) and (n0 + 2, n0 + 3), n0 % 4 == 0: all
-// population and module boundaries (250, 1000, 1250) are even.
-__device__ __forceinline__ void pair_pops(uint32_t n0, int &p0, int &p1) {
-  const uint32_t l0 = n0 % (uint32_t)kK;
-  const uint32_t l1 = (l0 + 2u == (uint32_t)kK) ? 0u : l0 + 2u;
-  p0 = pop_of_local(l0);
-  p1 = pop_of_local(l1);
-}
-
-// Number of thresholds <= u (thresholds ascend), u = w >> 12.
-__device__ __forceinline__ uint32_t events_of(const NetDev &nd, int pop, const uint4 &th, uint32_t w) {
-  const uint32_t u = w >> 12;
-  uint32_t k = (u >= th.x ? 1u : 0u) + (u >= th.y ? 1u : 0u) + (u >= th.z ? 1u : 0u);
-  if (u >= th.w) {
-    k = 4u;
-    while (k < (uint32_t)kPoisMax && u >= nd.thr[pop][k]) ++k;
-  }
-  return k;
-}
-
-// External drive of 4 neurons at step t without the events after each neuron's
-// first (kx counts them all).
-__device__ __forceinline__ int4 first_drive(const NetDev &nd, uint32_t n0, uint32_t t, int p0, int p1, uint32_t (&kx)[4]) {
-  const uint4 R = philox4x32_10(n0 >> 2, t, 1u, 0u, nd.key0, nd.key1);
-  const uint4 t0 = *reinterpret_cast<const uint4 *>(nd.thr[p0]);
-  const uint4 t1 = *reinterpret_cast<const uint4 *>(nd.thr[p1]);
-  kx[0] = events_of(nd, p0, t0, R.x);
-  kx[1] = events_of(nd, p0, t0, R.y);
-  kx[2] = events_of(nd, p1, t1, R.z);
-  kx[3] = events_of(nd, p1, t1, R.w);
-  const int32_t *a0 = nd.amp + p0 * kZTab, *a1 = nd.amp + p1 * kZTab;
-  int4 I = make_int4(0, 0, 0, 0);
-  if (kx[0]) I.x = __ldg(a0 + (R.x & 0xFFFu));
-  if (kx[1]) I.y = __ldg(a0 + (R.y & 0xFFFu));
-  if (kx[2]) I.z = __ldg(a1 + (R.z & 0xFFFu));
-  if (kx[3]) I.w = __ldg(a1 + (R.w & 0xFFFu));
-  return I;
-}
-
-// Eq. 2 over one step (the operations and roundings of neuron_step, without branches).
-__device__ __forceinline__ bool run_step(const float4 &pa, const float4 &pb, float &V, float &c, uint32_t &ref, int32_t I,
-                                         bool live) {
-  const float c_old = c;
-  const float b = __fmul_rn(pa.x, __fsub_rn(V, pa.w));
-  const float f = __fadd_rn(b, __fmul_rn(pa.y, c_old));
-  const float g = __fadd_rn(pa.w, f);
-  const float vn = __fadd_rn(g, __fmul_rn(__int2float_rn(I), 1.0f / 65536.0f));
-  const bool held = ref > 0u;
-  const bool spike = live && !held && vn > pb.x;
-  V = (held || spike) ? pb.y : vn;
-  ref = held ? ref - 1u : (spike ? __float_as_uint(pb.w) : 0u);
-  float cn = __fmul_rn(pa.z, c_old);
-  if (spike) cn = __fadd_rn(cn, pb.z);
-  c = cn;
-  return spike;
-}
-
-__device__ __forceinline__ uint32_t run_step4(const NetDev &nd, uint32_t n0, int p0, int p1, float4 &V, float4 &c, uint32_t &ref,
-                                              const int4 &I) {
-  const float4 a0 = nd.pa[p0], b0 = nd.pb[p0], a1 = nd.pa[p1], b1 = nd.pb[p1];
-  uint32_t r0 = ref & 0xFFu, r1 = (ref >> 8) & 0xFFu, r2 = (ref >> 16) & 0xFFu, r3 = ref >> 24;
-  const bool l0 = n0 < nd.N, l1 = n0 + 2u < nd.N;   // N is even
-  uint32_t mask = 0;
-  if (run_step(a0, b0, V.x, c.x, r0, I.x, l0)) mask |= 1u;
-  if (run_step(a0, b0, V.y, c.y, r1, I.y, l0)) mask |= 2u;
-  if (run_step(a1, b1, V.z, c.z, r2, I.z, l1)) mask |= 4u;
-  if (run_step(a1, b1, V.w, c.w, r3, I.w, l1)) mask |= 8u;
-  ref = r0 | (r1 << 8) | (r2 << 16) | (r3 << 24);
-  return mask;
-}
-
 // Forms of the kernel (all networks of a launch have the same smallest delay
 // kmin, and the same phase of its period).
 //   kAhead   kmin = 1.  After step k the spikes of steps k, k - visit,
