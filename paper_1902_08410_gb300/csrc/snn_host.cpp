@@ -402,8 +402,8 @@ struct snn_net {
 // a state of up to kSmallState bytes is read in one copy through pinned memory,
 // not in three pageable ones.  One step of 5000 neurons: 37 -> 28 us, the read
 // of its state 29 -> 13 us.
-// Longer windows and larger states gain nothing measurable: one more copy a
-// window, one more pass over the state.
+// Longer windows fetch their entries while the GPU runs the next one; larger
+// states would need a larger pinned buffer in every network.
 constexpr uint64_t kHeadSteps = 16;
 constexpr uint32_t kHeadEntries = 64;
 constexpr size_t kSmallState = 64 * 1024;
@@ -458,8 +458,12 @@ static void l2_release(snn_net *h) {
 // 80; 90-98 with V, c and ref alone in the window, 110-120 with the
 // set-aside raised and no window; 3.92M neurons, which fit: 57 in it, 61 without).
 // The spike lists (sparse: only the ids of recent spikes are touched) are never
-// part of it.
-static size_t l2_window_bytes(const snn_net *h) {
+// part of it.  The persistent kernel (`part` 4) takes one up to a quarter of the
+// set-aside only: it reads V, c and ref once a window, and of its six input
+// buffers the window holds two (us a step with and without: 16 modules 3.34 and
+// 3.38, 64 to 900 within 1%, 1156 16.8 and 16.6, 1444 24.1 and 22.9, 1600 27.2
+// and 24.7).
+static size_t l2_window_bytes(const snn_net *h, size_t part) {
   int dev = 0, max_win = 0, max_persist = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&max_win, cudaDevAttrMaxAccessPolicyWindowSize, dev) != cudaSuccess ||
@@ -468,17 +472,17 @@ static size_t l2_window_bytes(const snn_net *h) {
     return 0;
   }
   const size_t all = h->L.off_hist;
-  return all <= (size_t)max_persist ? std::min<size_t>(all, (size_t)max_win) : 0;
+  return all <= (size_t)max_persist / part ? std::min<size_t>(all, (size_t)max_win) : 0;
 }
 
 // The persisting window of network h.  Networks that run at the same time
 // keep their full hit ratio: splitting the set-aside between two 24x24
 // networks (ratio 0.63 each) was 10% slower than letting their persisting
 // lines compete.
-static int l2_window(snn_net *h, L2Window *out) {
+static int l2_window(snn_net *h, L2Window *out, size_t part = 1) {
   *out = L2Window{};
   if (!h->cfg.l2_persist) return SNN_OK;
-  const size_t bytes = l2_window_bytes(h);
+  const size_t bytes = l2_window_bytes(h, part);
   if (bytes == 0) return SNN_OK;
   int rc = l2_acquire(h);
   if (rc) return rc;
@@ -1021,7 +1025,7 @@ static int runner_start(PlainRunner &r, snn_net *h, uint64_t steps) {
   r.t_issue = h->t;
   if (!steps) return SNN_OK;
   r.shape = plain_shape(h);
-  return r.shape.blocks > 0 ? l2_window(h, &r.l2) : prepare_graphs(h, r.window);
+  return r.shape.blocks > 0 ? l2_window(h, &r.l2, 4) : prepare_graphs(h, r.window);
 }
 
 static int run_plain(snn_net *h, uint64_t steps) {

@@ -21,10 +21,10 @@
 //     of its new spikes stand between two barriers.
 //
 // What bounds it: small networks, the grid barrier and two L2 or DRAM round trips
-// a step (4x4 modules: 5.3 us a step as two kernels, 2.9 us here); larger ones,
+// a step (4x4 modules: 5.3 us a step as two kernels, 2.5 us here); larger ones,
 // the visits' reductions, about 3e11 a second in L2, beside the issue of update
 // and drive (24x24 modules at 8.7 Hz: 17.8 us as two kernels in the default
-// shape, 11.9 us here; 64 networks of 2.3M neurons in all: 78 us as one kernel
+// shape, 11.3 us here; 64 networks of 2.3M neurons in all: 78 us as one kernel
 // per step, 53 us here).  Measured beside it: one delay group per visit, 13-15 us
 // at 24x24; whole modules per block with the records of the own module summed in
 // shared memory, 17 us (blocks whose modules are active hold up the grid).
@@ -796,7 +796,7 @@ cudaError_t prepare_run_kernels() {
 // 512: 8% more from 16x16 on) but fewer for a few tiles, where the block barriers
 // cost more than further warps give.  The form fits as long as the state and `kmin` drives per
 // neuron stay in shared memory (2.1M neurons at kmin = 1); what does not fit
-// takes two kernels per step (64x64 modules: 105 us a step, against 125 and 217 us
+// takes two kernels per step (64x64 modules: 80 us a step, against 125 and 217 us
 // in two forms of this kernel with the state in global memory).
 RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads) {
   RunShape sh;
