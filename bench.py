@@ -221,8 +221,11 @@ def measured_peaks() -> tuple[float, str]:
 
 
 def kernel_source_hash() -> str:
-    with open(os.path.join(ROOT, "paper_1902_08410_gb300", "csrc", "snn_kernels.cu"), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in ("snn_device.cuh", "snn_kernels.cu"):
+        with open(os.path.join(ROOT, "paper_1902_08410_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def committed_traffic(kernel: str) -> float | None:
@@ -366,8 +369,8 @@ def run_gb300(args, dist: Dist):
         names.append(reg)
     # Two ways to advance the pair: "concurrent" (two-kernel path, each network
     # tuned alone, then the pair tuned running together, each on its own
-    # stream) and "batch" (both networks in one fused kernel per step, shape
-    # tuned on the pair).  After the initial volley both are tuned and timed on
+    # stream) and "batch" (a window of both networks in one launch of the
+    # persistent kernel, shape tuned on the pair).  After the initial volley both are tuned and timed on
     # alternating stretches of the same run; the faster one is benchmarked.
     form, form_trial = ("sequential" if args.sequential else "concurrent"), None
     if not args.no_tune:
@@ -501,16 +504,16 @@ def run_gb300(args, dist: Dist):
               f"steps apart, each as a graph timed with CUDA events) x the kernel's share of the same steps run "
               f"again with event nodes; delivery bytes = timed-region spikes per step x (M x record bytes + 8)")
     if form == "batch":
-        # the timed region ran one fused kernel per step for both networks:
-        # its launch duration is the timed region's time per step
+        # the timed region ran both networks in one launch of the persistent
+        # kernel per window: its figures are the timed region's per step
         fu_ms = 1e3 * elapsed / (args.steps * steps)
         fu_b = sum(x["update_bytes"] + x["deliver_bytes"] for x in per_net)
-        kernels["k_fused"] = {"ms_per_launch": fu_ms, "algorithmic_bytes": fu_b,
+        kernels["k_run"] = {"ms_per_launch": fu_ms, "algorithmic_bytes": fu_b,
                               "achieved_gbs": fu_b / (fu_ms * 1e-3) / 1e9}
-        share["k_fused"] = 1.0
-        dom = "k_fused"
-        method = ("k_fused: one launch per step for both networks in the timed region; launch duration = timed "
-                  "region / steps (CUDA events on the launching stream), bytes = both networks' neuron state + "
+        share["k_run"] = 1.0
+        dom = "k_run"
+        method = ("k_run: one launch per window for both networks in the timed region; ms_per_launch = timed "
+                  "region / steps (CUDA events on the launching stream; one step of a launch), bytes = both networks' neuron state + "
                   "timed-region spikes per step x (M x record bytes + 8).  k_update / k_deliver: the two-kernel "
                   "path of each network alone, for reference (" + method + ")")
     ach = kernels[dom]["achieved_gbs"]
@@ -612,7 +615,7 @@ def run_gb300(args, dist: Dist):
                                         "concurrent": "concurrently, one CUDA stream each, two-kernel path "
                                                       "(snn_run_concurrent), shapes tuned with both running "
                                                       "(snn_autotune_concurrent)",
-                                        "batch": "together, one fused kernel per step for both networks "
+                                        "batch": "together, one launch per window for both networks "
                                                  "(snn_run_batch)"}[form],
                        "form_trial": form_trial},
             "sim_seconds_per_wall_second": sim_s * len(nets) * dist.world / t_max,
@@ -628,14 +631,14 @@ def run_gb300(args, dist: Dist):
 
 
 # ---------------------------------------------------------------------------
-# batched sweep: one fused kernel per step over all networks vs one network per launch
+# batched sweep: one launch per window over all networks vs one network per launch
 # ---------------------------------------------------------------------------
 def measure_batch(snn, torch, dist: Dist, n_nets: int, warm: int, timed: int, plain_timed: int,
                   plain_nets: int | None = None) -> tuple[dict, list, list]:
-    """The batched sweep: `n_nets` networks on the fused path (one kernel per
-    step for all of them, shape from the batch tuner after `warm` steps), then
-    `timed` steps timed; beside it one network per launch (two kernels per
-    step, each network alone) on fresh copies of the first `plain_nets`
+    """The batched sweep: `n_nets` networks in one launch per window for all
+    of them (shape from the batch tuner after `warm` steps), then `timed` steps
+    timed; beside it one network per launch (each network alone, in the
+    default shape) on fresh copies of the first `plain_nets`
     networks: their first `warm` steps compared with the batch's rasters, the
     next `plain_timed` steps timed.  Returns (result, specs, batch networks)."""
     import numpy as np
@@ -647,7 +650,7 @@ def measure_batch(snn, torch, dist: Dist, n_nets: int, warm: int, timed: int, pl
     for n in nets:
         n.launch = {"path": 1}
     stream = torch.cuda.current_stream()
-    # the first steps (the initial volley) untimed, then the fused shape tuned
+    # the first steps (the initial volley) untimed, then the shape tuned
     # on the whole batch (state restored after the trials)
     snn.run_batch(nets, [warm] * len(nets))
     tuned = snn.autotune_batch(nets, 200)
