@@ -959,7 +959,7 @@ struct PlainRunner {
 static RunShape plain_shape(const snn_net *h) {
   if (h->cfg.path == 0 && !has_default_shape(h->cfg)) return RunShape{};
   const int threads = h->cfg.path == 1 ? h->cfg.fused_block * h->cfg.fused_items_per_sm : 1024;
-  return run_shape(h->L.N_pad / 128u, h->L.kmin, std::min(threads, 1024));
+  return run_shape(h->L.N_pad / 128u, h->L.kmin, std::min(threads, 1024), 1u);
 }
 
 static uint32_t plain_window(const snn_net *h) {
@@ -1231,7 +1231,7 @@ static int run_set(snn_net *const *hs, const uint64_t *steps, int32_t n) {
     uint64_t tiles = 0;
     while (at < n && (g.empty() || key(order[at]) == std::make_pair(g[0]->L.kmin, g[0]->t % g[0]->L.kmin))) {
       snn_net *h = hs[order[at]];
-      const RunShape next = run_shape((uint32_t)(tiles + h->L.N_pad / 128u), h->L.kmin, threads);
+      const RunShape next = run_shape((uint32_t)(tiles + h->L.N_pad / 128u), h->L.kmin, threads, (uint32_t)g.size() + 1u);
       if (next.blocks < 1 && !g.empty()) break;
       g.push_back(h);
       st.push_back(steps[order[at]]);

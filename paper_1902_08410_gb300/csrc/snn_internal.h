@@ -160,10 +160,11 @@ struct RunShape {
   int blocks = 0, threads = 0;
   int form = 0;               // RunForm
   uint32_t fifo = 0, nt = 0, visit = 1, drives = 1;
+  uint32_t tables = 0;        // networks whose descriptors fit in shared memory beside the rest
   size_t smem = 0;
 };
 // blocks == 0: too many tiles for one launch.
-RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads);
+RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_nets);
 cudaError_t launch_run(const RunArgs &a, const RunShape &sh, const L2Window &l2, cudaStream_t s);
 cudaError_t prepare_run_kernels();
 // Delivery keeps each warp's segment prefix in registers, in chunks of 32

@@ -83,14 +83,21 @@ struct RunShared {
   Pending pend[2];
 };
 
-template <bool MULTI>
-__device__ __forceinline__ const NetDev &net_of(const RunArgs &a, const RunShared &s, uint32_t net) {
-  if constexpr (MULTI) return a.nets[net];
+// MULTI: one network (its descriptor a kernel parameter), several, or several
+// whose descriptors are copied to shared memory.  From global memory every
+// interval reads them anew, a round trip per tile and visit: 16 networks of 4x4
+// modules 8.2 us a step, 7.5 from shared memory; 4 of 16x16 21.7, 20.1; a batch
+// that leaves no room for them is 2% faster with a kernel of its own.
+enum RunNets : int { kOne = 0, kSeveral = 1, kTables = 2 };
+
+template <int MULTI>
+__device__ __forceinline__ const NetDev &net_of(const NetDev *nets, const RunShared &s, uint32_t net) {
+  if constexpr (MULTI) return nets[net];
   else return s.nd;
 }
-template <bool MULTI>
-__device__ __forceinline__ NetWin win_of(const RunArgs &a, uint32_t net) {
-  if constexpr (MULTI) return a.wins[net];
+template <int MULTI>
+__device__ __forceinline__ NetWin win_of(const RunArgs &a, const NetWin *wins, uint32_t net) {
+  if constexpr (MULTI) return wins[net];
   else return a.win;
 }
 __device__ __forceinline__ bool pass_after(const NetDev &nd, uint32_t t) { return nd.kmin == 1u || (t + 1u) % nd.kmin == 0u; }
@@ -254,7 +261,7 @@ static __device__ __noinline__ void deliver_lists(const NetDev &nd, uint32_t t, 
 }
 
 // Network and first neuron of tile g of the table.
-template <bool MULTI>
+template <int MULTI>
 __device__ __forceinline__ uint2 tile_at(const RunArgs &a, uint32_t g) {
   if constexpr (!MULTI) return make_uint2(0u, g * 128u);
   uint32_t lo = 0, hi = a.n_nets;   // last network with tile_pre <= g
@@ -290,7 +297,7 @@ struct Width {
 };
 
 // MULTI: several networks (device tables).
-template <bool MULTI, int FORM>
+template <int MULTI, int FORM>
 __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ RunArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ RunShared s;
@@ -309,12 +316,21 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   float4 *s_c = s_V + a.nt * 32u;
   uint32_t *s_ref = reinterpret_cast<uint32_t *>(s_c + a.nt * 32u);
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = lane_id(), nw = blockDim.x >> 5;
+  // descriptors and windows of several networks, in shared memory where they fit: a barrier ends what L1 holds of them
+  const NetDev *nets = MULTI == kTables ? reinterpret_cast<const NetDev *>(s_ref + a.nt * 32u) : a.nets;   // 16-byte aligned
+  const NetWin *wins = MULTI == kTables ? reinterpret_cast<const NetWin *>(nets + a.n_nets) : a.wins;
 
   // ---- prologue
   if constexpr (!MULTI) {
     const uint32_t *src = reinterpret_cast<const uint32_t *>(&a.nd);
     uint32_t *dst = reinterpret_cast<uint32_t *>(&s.nd);
     for (uint32_t i = tid; i < sizeof(NetDev) / 4; i += blockDim.x) dst[i] = src[i];
+  }
+  if constexpr (MULTI == kTables) {
+    uint4 *dst = reinterpret_cast<uint4 *>(s_ref + a.nt * 32u);
+    const uint32_t n = a.n_nets * (uint32_t)(sizeof(NetDev) / 16u), m = a.n_nets * (uint32_t)(sizeof(NetWin) / 16u);
+    for (uint32_t i = tid; i < n + m; i += blockDim.x)
+      dst[i] = i < n ? reinterpret_cast<const uint4 *>(a.nets)[i] : reinterpret_cast<const uint4 *>(a.wins)[i - n];
   }
   if (tid == 0) {
     for (uint32_t c = 0; c < kMaxVisit; ++c) s.tail[c] = s.base[c] = s.head[c] = 0u;
@@ -332,7 +348,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   __syncthreads();
   for (uint32_t j = warp; j < nt; j += nw) {
     const uint2 tile = s_tile[j];
-    const NetDev &nd = net_of<MULTI>(a, s, tile.x);
+    const NetDev &nd = net_of<MULTI>(nets, s, tile.x);
     const uint32_t i4 = (tile.y >> 2) + lane;
     s_V[j * 32u + lane] = ld_cg_f4(reinterpret_cast<const float4 *>(nd.V) + i4);
     s_c[j * 32u + lane] = ld_cg_f4(reinterpret_cast<const float4 *>(nd.c) + i4);
@@ -347,8 +363,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   auto each_slot = [&](auto &&use) {
     for (uint32_t i = tid; i < a.n_nets * a.nd_max; i += blockDim.x) {
       const uint32_t net = MULTI ? i / a.nd_max : 0u, back = i - net * a.nd_max + 1u;   // step t0 - back
-      const NetDev &nd = net_of<MULTI>(a, s, net);
-      const NetWin w = win_of<MULTI>(a, net);
+      const NetDev &nd = net_of<MULTI>(nets, s, net);
+      const NetWin w = win_of<MULTI>(a, wins, net);
       if (w.t0 >= w.t_end || back > w.t0) continue;
       const uint32_t tp = w.t0 + (nd.kmin - 1u - w.t0 % nd.kmin);   // first pass of the window
       if (tp + 1u > w.t0 - back + nd.n_delay) continue;
@@ -394,8 +410,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
         int kts;
         live_unpack(live[c * cap + (e & (cap - 1u))], id, kts, p, net);
         if (kts < 0) continue;   // in the lists already
-        const NetDev &nd = net_of<MULTI>(a, s, net);
-        const NetWin w = win_of<MULTI>(a, net);
+        const NetDev &nd = net_of<MULTI>(nets, s, net);
+        const NetWin w = win_of<MULTI>(a, wins, net);
         const uint32_t adv = w.t_end - w.t0;
         if (adv >= lo && adv <= hi && w.t0 + (uint32_t)kts + nd.n_delay >= w.t_end)
           list_append(nd, w.t0 + (uint32_t)kts, id);
@@ -403,7 +419,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   };
   auto find_end = [&](uint32_t k) {
     for (uint32_t i = tid; i < a.n_nets; i += blockDim.x) {
-      const uint32_t adv = a.wins[i].t_end - a.wins[i].t0;
+      const uint32_t adv = wins[i].t_end - wins[i].t0;
       if (adv > k && adv < a.steps) atomicMin(&s.end_k, adv);
     }
   };
@@ -423,8 +439,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     uint32_t id, p, net;
     int kts;
     live_unpack(*at, id, kts, p, net);
-    const NetDev &nd = net_of<MULTI>(a, s, net);
-    const NetWin w = win_of<MULTI>(a, net);
+    const NetDev &nd = net_of<MULTI>(nets, s, net);
+    const NetWin w = win_of<MULTI>(a, wins, net);
     const uint32_t adv = w.t_end - w.t0;
     // kAhead: nothing beyond the first step after the network's window
     const int dlim = (int)(PERIOD ? upto : min(upto, adv)) - kts;
@@ -456,8 +472,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
       if (u >= units) break;
       const uint32_t i = PERIOD ? u / nt : 0u, j = PERIOD ? u - i * nt : u;
       const uint2 tile = s_tile[j];
-      const NetDev &nd = net_of<MULTI>(a, s, tile.x);
-      const NetWin w = win_of<MULTI>(a, tile.x);
+      const NetDev &nd = net_of<MULTI>(nets, s, tile.x);
+      const NetWin w = win_of<MULTI>(a, wins, tile.x);
       const uint32_t t = w.t0 + k + i;
       if (t >= w.t_end) continue;
       const uint32_t n0 = tile.y + lane * 4u, slot = PERIOD ? j * P + i : (deep ? j * 2u + (k & 1u) : j);
@@ -492,10 +508,10 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
       const uint32_t e = pend.list[x], at = e >> 5, kx = e & 31u;
       const uint32_t slot = at >> 7, j = PERIOD ? slot / P : slot >> (deep ? 1 : 0), i = PERIOD ? slot - j * P : 0u;
       const uint2 tile = s_tile[j];
-      const NetDev &nd = net_of<MULTI>(a, s, tile.x);
+      const NetDev &nd = net_of<MULTI>(nets, s, tile.x);
       const uint32_t n = tile.y + (at & 127u);
       reinterpret_cast<int32_t *>(s_I)[at] +=
-          extra_sum(nd, pop_of_local(n % (uint32_t)kK), kx, n, win_of<MULTI>(a, tile.x).t0 + k + i);
+          extra_sum(nd, pop_of_local(n % (uint32_t)kK), kx, n, win_of<MULTI>(a, wins, tile.x).t0 + k + i);
     }
   };
   const uint32_t phase0 = PERIOD ? (MULTI ? a.wins[0].t0 : a.win.t0) % a.kmin : 0u;
@@ -535,8 +551,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     // the list counts of the steps after a pass start at zero (not read or appended to before the next barrier)
     if (warp == nw - 1u)
       for (uint32_t net = blockIdx.x + lane * gridDim.x; net < a.n_nets; net += gridDim.x * 32u) {
-        const NetDev &nd = net_of<MULTI>(a, s, net);
-        const NetWin w = win_of<MULTI>(a, net);
+        const NetDev &nd = net_of<MULTI>(nets, s, net);
+        const NetWin w = win_of<MULTI>(a, wins, net);
         const uint32_t t = w.t0 + kl;
         if (t < w.t_end && pass_after(nd, t))
           for (uint32_t i = 0; i < nd.kmin; ++i) nd.cnt[(t + 1u + i) % nd.D] = 0u;
@@ -545,8 +561,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     // ---- update of the block's tiles
     for (uint32_t j = warp; j < nt; j += nw) {
       const uint2 tile = s_tile[j];
-      const NetDev &nd = net_of<MULTI>(a, s, tile.x);
-      const NetWin w = win_of<MULTI>(a, tile.x);
+      const NetDev &nd = net_of<MULTI>(nets, s, tile.x);
+      const NetWin w = win_of<MULTI>(a, wins, tile.x);
       if (w.t0 + k >= w.t_end) continue;
       const uint32_t n0 = tile.y + lane * 4u, i4 = n0 >> 2;
       constexpr uint32_t IN = PERIOD ? 4u : 1u;   // steps whose inputs are loaded together
@@ -663,7 +679,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
         while (net > 0u && max(first(net - 1u) + 1u, first(net)) > gw) --net;   // the first network with this warp
         for (; net < a.n_nets && first(net) <= gw; ++net) {
           const uint32_t lo = first(net), hi = max(lo + 1u, first(net + 1u));
-          if (hi > gw) lists(a.nets[net], a.wins[net], gw - lo, hi - lo);
+          if (hi > gw) lists(nets[net], wins[net], gw - lo, hi - lo);
         }
       }
     }
@@ -693,12 +709,12 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
         if (e < tail) live_unpack(rlive[e & (cap - 1u)], id, kts, p, net);
         uint32_t at = 0;
         if constexpr (MULTI) {
-          if (e < tail) at = atomicAdd(&a.nets[net].rec->cursor, 1u);
+          if (e < tail) at = atomicAdd(&nets[net].rec->cursor, 1u);
         } else {
           if (lane == 0) at = atomicAdd(&s.nd.rec->cursor, min(32u, tail - e0));
           at = __shfl_sync(0xFFFFFFFFu, at, 0) + lane;
         }
-        if (e < tail) record_at(net_of<MULTI>(a, s, net), win_of<MULTI>(a, net), at, id, (uint32_t)kts);
+        if (e < tail) record_at(net_of<MULTI>(nets, s, net), win_of<MULTI>(a, wins, net), at, id, (uint32_t)kts);
       }
     }
     if constexpr (PERIOD) {
@@ -730,12 +746,12 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   leave(a.steps, a.steps);
   for (uint32_t j = tid; j < nt; j += blockDim.x) {
     const uint2 tile = s_tile[j];
-    if (s_ext[j]) net_of<MULTI>(a, s, tile.x).ext_acc[tile.y >> 7] += s_ext[j];
+    if (s_ext[j]) net_of<MULTI>(nets, s, tile.x).ext_acc[tile.y >> 7] += s_ext[j];
   }
   for (uint32_t j = warp; j < nt; j += nw) {
     const uint2 tile = s_tile[j];
-    const NetDev &nd = net_of<MULTI>(a, s, tile.x);
-    const NetWin w = win_of<MULTI>(a, tile.x);
+    const NetDev &nd = net_of<MULTI>(nets, s, tile.x);
+    const NetWin w = win_of<MULTI>(a, wins, tile.x);
     const uint32_t n0 = tile.y + lane * 4u, i4 = n0 >> 2;
     if (n0 >= nd.N) continue;
     if constexpr (!PERIOD) {   // the input of the next step goes where the other paths read it
@@ -776,15 +792,16 @@ static size_t run_smem_budget() {
 
 using RunKernel = void (*)(RunArgs);
 
-static RunKernel run_kernel(bool multi, int form) {
-  if (form == kPeriod) return multi ? k_run<true, kPeriod> : k_run<false, kPeriod>;
-  return multi ? k_run<true, kAhead> : k_run<false, kAhead>;
+static RunKernel run_kernel(int nets, int form) {
+  if (form == kPeriod)
+    return nets == kOne ? k_run<kOne, kPeriod> : (nets == kSeveral ? k_run<kSeveral, kPeriod> : k_run<kTables, kPeriod>);
+  return nets == kOne ? k_run<kOne, kAhead> : (nets == kSeveral ? k_run<kSeveral, kAhead> : k_run<kTables, kAhead>);
 }
 
 cudaError_t prepare_run_kernels() {
-  for (bool multi : {false, true})
+  for (int nets : {kOne, kSeveral, kTables})
     for (int form : {kAhead, kPeriod}) {
-      cudaError_t e = cudaFuncSetAttribute(run_kernel(multi, form), cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaError_t e = cudaFuncSetAttribute(run_kernel(nets, form), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)run_smem_budget());
       if (e != cudaSuccess) return e;
     }
@@ -798,7 +815,7 @@ cudaError_t prepare_run_kernels() {
 // neuron stay in shared memory (2.1M neurons at kmin = 1); what does not fit
 // takes two kernels per step (64x64 modules: 80 us a step, against 125 and 217 us
 // in two forms of this kernel with the state in global memory).
-RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads) {
+RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_nets) {
   RunShape sh;
   const uint32_t sms = (uint32_t)std::max(1, device_sm_count());
   sh.blocks = (int)std::max(1u, std::min(sms, n_tiles));
@@ -812,8 +829,12 @@ RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads) {
   // Drives a step further ahead where they fit: the neurons with several external events are then completed beside
   // the visits instead of behind a block barrier.
   sh.drives = sh.form == kPeriod ? kmin : (run_smem(2u, sh.nt, sh.visit * sh.fifo) <= budget ? 2u : 1u);
-  while (sh.fifo < 8192u / sh.visit && run_smem(sh.drives, sh.nt, sh.visit * sh.fifo * 2u) <= budget) sh.fifo *= 2u;
-  sh.smem = run_smem(sh.drives, sh.nt, sh.visit * sh.fifo);
+  const size_t tables = n_nets > 1u ? n_nets * (sizeof(NetDev) + sizeof(NetWin)) : 0u;
+  sh.tables = tables && run_smem(sh.drives, sh.nt, sh.visit * sh.fifo) + tables <= budget ? n_nets : 0u;
+  const size_t fixed = sh.tables ? tables : 0u;
+  while (sh.fifo < 8192u / sh.visit && run_smem(sh.drives, sh.nt, sh.visit * sh.fifo * 2u) + fixed <= budget)
+    sh.fifo *= 2u;
+  sh.smem = run_smem(sh.drives, sh.nt, sh.visit * sh.fifo) + fixed;
   if (sh.smem > budget) sh.blocks = 0;   // too many tiles per block
   return sh;
 }
@@ -826,6 +847,7 @@ cudaError_t launch_run(const RunArgs &args, const RunShape &sh, const L2Window &
   a.nt = sh.nt;
   a.visit = sh.visit;
   a.drives = sh.drives;
+  const int nets = a.n_nets < 2u ? kOne : (sh.tables >= a.n_nets ? kTables : kSeveral);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)sh.blocks);
   cfg.blockDim = dim3((unsigned)sh.threads);
@@ -846,7 +868,7 @@ cudaError_t launch_run(const RunArgs &args, const RunShape &sh, const L2Window &
   }
   cfg.attrs = attr;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, run_kernel(a.n_nets > 1u, sh.form), a);
+  return cudaLaunchKernelEx(&cfg, run_kernel(nets, sh.form), a);
 }
 
 }  // namespace snn
