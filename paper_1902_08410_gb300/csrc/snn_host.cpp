@@ -1258,7 +1258,7 @@ static int run_set(snn_net *const *hs, const uint64_t *steps, int32_t n) {
 constexpr uint32_t kApartNeurons = 500000;
 
 static bool run_apart(snn_net *const *hs, const uint64_t *steps, int32_t n) {
-  if (n != 2) return false;
+  if (n != 2 || hs[0]->stream == hs[1]->stream) return false;   // on one stream they would take turns
   for (int i = 0; i < n; ++i)
     if (hs[i]->L.N < kApartNeurons || hs[i]->L.kmin != 1u || steps[i] < 2u * (uint64_t)plain_window(hs[i])) return false;
   return true;
