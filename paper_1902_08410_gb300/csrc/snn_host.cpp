@@ -983,6 +983,7 @@ static int runner_issue(PlainRunner &r) {
     a.steps = (uint32_t)n;
     a.nd_max = (uint32_t)h->p.n_delay;
     a.kmin = h->L.kmin;
+    a.phase = a.win.t0 % a.kmin;
     // the barrier words follow the header in the recording block, which is zero at every window start
     a.bar = reinterpret_cast<uint32_t *>(base + h->L.off_rec[b] + 128);
     a.status = &a.nd.rec->status;
@@ -1183,8 +1184,11 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
       a.steps = (uint32_t)std::min<uint64_t>(window, most);
       a.nd_max = nd_max;
       a.kmin = hs[0]->L.kmin;
-      int first = 0;   // a network that advances: its recording block is copied and checked
+      // a network that advances: its recording block is copied and checked, and the exchange periods of all that
+      // advance are counted from its first step (one that has stopped keeps the step, and phase, of its end)
+      int first = 0;
       while (!p.adv[first]) ++first;
+      a.phase = (uint32_t)(p.t0s[first] % a.kmin);
       a.status = &reinterpret_cast<const NetDev *>(B.pinned[b])[first].rec->status;
       CU_TRY(launch_run(a, shape, L2Window{}, s));
       ++hs[0]->launches;

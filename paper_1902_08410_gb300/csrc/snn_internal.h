@@ -147,6 +147,7 @@ struct RunArgs {
   uint32_t steps;             // steps of the window (the longest of the networks)
   uint32_t nd_max;            // largest delay of the networks
   uint32_t kmin;              // smallest delay, the same for all networks
+  uint32_t phase;             // t0 mod kmin, the same for all networks that advance (those that have stopped: any)
   uint32_t visit;             // steps between two visits of a live spike (1 in the period form)
   uint32_t fifo;              // live spikes of one ring that a block holds in shared memory (power of two)
   uint32_t nt;                // tiles of a block, at most

@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
           extra_sum(nd, pop_of_local(n % (uint32_t)kK), kx, n, win_of<MULTI>(a, wins, tile.x).t0 + k + i);
     }
   };
-  const uint32_t phase0 = PERIOD ? (MULTI ? a.wins[0].t0 : a.win.t0) % a.kmin : 0u;
+  const uint32_t phase0 = PERIOD ? a.phase : 0u;
   auto interval = [&](uint32_t k) {   // steps until the grid meets again
     return PERIOD ? min(a.kmin - (phase0 + k) % a.kmin, a.steps - k) : 1u;
   };

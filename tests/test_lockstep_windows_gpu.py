@@ -1,0 +1,52 @@
+"""Networks of unequal lengths in one launch per window, over several windows
+and calls: those that stop first, or do not advance at all, leave the others'
+exchange periods where they are."""
+import pytest
+
+import workloads as W
+from parity import assert_same, gpu_results, oracle_results
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("window", [12, 64])
+@pytest.mark.parametrize("min_delay,calls", [(10, [(105, 700, 333), (0, 41, 7), (50, 9, 320)]),
+                                             (3, [(10, 0, 200), (65, 130, 1)]), (1, [(10, 0, 200), (65, 130, 1)])])
+@pytest.mark.parametrize("run", ["run_batch", "run_concurrent"])
+def test_unequal_lengths(oracle_mod, min_delay, calls, window, run):
+    import paper_1902_08410_gb300 as snn
+    nets, params = [], []
+    for i, (gx, gy) in enumerate(((1, 1), (3, 2), (2, 1))):
+        p = W.base_params(gx, gy, 0.7, "AW", record_format=i % 2)
+        p["min_delay"] = min_delay
+        params.append(p)
+        nets.append(snn.Network(p, 90 + i))
+        nets[i].launch = {"window_steps": window}
+    for steps in calls:
+        getattr(snn, run)(nets, steps)
+    for i, g in enumerate(nets):
+        n = sum(c[i] for c in calls)
+        o = oracle_mod.OracleNet(params[i], 90 + i)
+        o.run(n)
+        assert_same(gpu_results(g), oracle_results(o), n)
+        g.close()
+
+
+def test_server_with_exchange_periods():
+    """Served networks of one smallest delay that end at any step."""
+    import numpy as np
+    import paper_1902_08410_gb300 as snn
+    from paper_1902_08410_gb300.serve import Server
+    p = dict(W.base_params(2, 2, 0.7, "AW"), min_delay=10)
+    lengths = [1205, 3300, 2777, 600]
+    srv = Server(memory_budget=8 << 30, chunk_steps=2500, realtime=False)
+    for i, n in enumerate(lengths):
+        srv.submit(p, 20 + i, n)
+    out = srv.run()["results"]
+    for i, n in enumerate(lengths):
+        g = snn.Network(p, 20 + i)
+        g.run(n)
+        st, ids = g.spikes()
+        assert len(st) and np.array_equal(out[i].spike_steps, st) and np.array_equal(out[i].spike_ids, ids)
+        assert np.array_equal(out[i].rates, g.rates())
+        g.close()
