@@ -937,7 +937,7 @@ static int drain_batch(snn_net *const *hs, int b, const uint64_t *t0s, const uin
   return SNN_OK;
 }
 
-// Windows of one network on the two-kernel path.  They alternate between the
+// Windows of one network (persistent kernel or two kernels per step).  They alternate between the
 // two buffer sets; up to two are in flight, and the host drains the older one
 // while the GPU runs the newer.
 struct PlainRunner {
@@ -1001,12 +1001,12 @@ static int runner_issue(PlainRunner &r) {
     h->h2d += sizeof(NetWin);
     h->launches += kernels;
   }
+  r.issued += n;
+  r.t_issue += n;
   rc = drain_copy_block(h, b, n, h->stream);
   if (rc) return rc;
   r.q[r.nq++] = PlainRunner::Pending{b, t0, n};
   r.next_b ^= 1;
-  r.issued += n;
-  r.t_issue += n;
   return SNN_OK;
 }
 
@@ -1029,13 +1029,21 @@ static int runner_start(PlainRunner &r, snn_net *h, uint64_t steps) {
   return r.shape.blocks > 0 ? l2_window(h, &r.l2, 4) : prepare_graphs(h, r.window);
 }
 
+// After a failure: nothing left in flight, and a network with a window that was
+// issued but not drained is invalid (its device state is ahead of the host's
+// records, or lost with the kernel).
+static void runner_failed(PlainRunner &r) {
+  cudaStreamSynchronize(r.h->stream);
+  if (r.t_issue != r.h->t) r.h->broken = true;
+}
+
 static int run_plain(snn_net *h, uint64_t steps) {
   PlainRunner r;
   int rc = runner_start(r, h, steps);
   if (rc) return rc;
   int status = SNN_OK;
   while (status == SNN_OK && r.busy()) status = r.can_issue() ? runner_issue(r) : runner_drain(r);
-  if (status != SNN_OK) cudaStreamSynchronize(h->stream);   // nothing left in flight
+  if (status != SNN_OK) runner_failed(r);
   return status;
 }
 
@@ -1059,7 +1067,7 @@ static int run_plain_many(snn_net *const *hs, const uint64_t *steps, int32_t n) 
     for (int i = 0; i < n; ++i) any |= rs[i].busy();
   }
   if (status != SNN_OK)
-    for (int i = 0; i < n; ++i) cudaStreamSynchronize(hs[i]->stream);
+    for (auto &r : rs) runner_failed(r);
   return status;
 }
 
@@ -1153,69 +1161,78 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
   int nq = 0, next_b = 0;
   std::vector<uint64_t> left(steps, steps + n), t_issue(n);
   for (int i = 0; i < n; ++i) t_issue[i] = hs[i]->t;
-  int status = SNN_OK;
-  while (status == SNN_OK) {
-    uint64_t most = 0;
-    for (int i = 0; i < n; ++i) most = std::max(most, left[i]);
-    if (most > 0 && nq < 2) {
-      const int b = next_b;
-      NetWin *pw = reinterpret_cast<NetWin *>(B.pinned[b] + B.wins_at());   // free: its window has been drained
-      Pending p{b, std::vector<uint64_t>(n), std::vector<uint64_t>(n)};
-      for (int i = 0; i < n; ++i) {
-        const uint64_t adv = std::min<uint64_t>(window, left[i]);
-        if (t_issue[i] + adv > 0xFFFFFFFFull) {
-          status = fail(SNN_ERR_LIMIT, "step counter beyond 2^32");
-          break;
-        }
-        set_window(hs[i], pw + i, t_issue[i], t_issue[i] + adv);
-        p.t0s[i] = t_issue[i];
-        p.adv[i] = adv;
-      }
-      if (status != SNN_OK) break;
-      uint8_t *tab = static_cast<uint8_t *>(B.tab[b].p);
-      CU_TRY(cudaMemcpyAsync(tab, B.pinned[b], B.bytes(), cudaMemcpyHostToDevice, s));
-      RunArgs a{};
-      a.nets = reinterpret_cast<const NetDev *>(tab);
-      a.wins = reinterpret_cast<const NetWin *>(tab + B.wins_at());
-      a.tile_pre = reinterpret_cast<const uint32_t *>(tab + B.pre_at());
-      a.bar = reinterpret_cast<uint32_t *>(tab + B.bar_at());
-      a.n_nets = (uint32_t)n;
-      a.n_tiles = n_tiles;
-      a.steps = (uint32_t)std::min<uint64_t>(window, most);
-      a.nd_max = nd_max;
-      a.kmin = hs[0]->L.kmin;
-      // a network that advances: its recording block is copied and checked, and the exchange periods of all that
-      // advance are counted from its first step (one that has stopped keeps the step, and phase, of its end)
-      int first = 0;
-      while (!p.adv[first]) ++first;
-      a.phase = (uint32_t)(p.t0s[first] % a.kmin);
-      a.status = &reinterpret_cast<const NetDev *>(B.pinned[b])[first].rec->status;
-      CU_TRY(launch_run(a, shape, L2Window{}, s));
-      ++hs[0]->launches;
-      hs[0]->h2d += B.bytes();
-      for (int i = 0; i < n; ++i) {
-        if (p.adv[i]) {
-          int rc = drain_copy_block(hs[i], b, p.adv[i], s);
-          if (rc) return rc;
-        }
-        t_issue[i] += p.adv[i];
-        left[i] -= p.adv[i];
-      }
-      CU_TRY(cudaEventRecord(B.ev_block[b], s));
-      q[nq++] = std::move(p);
-      next_b ^= 1;
-      continue;
+  uint64_t most = 0;   // steps left of the network that has most
+  auto issue = [&]() -> int {
+    const int b = next_b;
+    NetWin *pw = reinterpret_cast<NetWin *>(B.pinned[b] + B.wins_at());   // free: its window has been drained
+    Pending p{b, std::vector<uint64_t>(n), std::vector<uint64_t>(n)};
+    for (int i = 0; i < n; ++i) {
+      const uint64_t adv = std::min<uint64_t>(window, left[i]);
+      if (t_issue[i] + adv > 0xFFFFFFFFull) return fail(SNN_ERR_LIMIT, "step counter beyond 2^32");
+      set_window(hs[i], pw + i, t_issue[i], t_issue[i] + adv);
+      p.t0s[i] = t_issue[i];
+      p.adv[i] = adv;
     }
-    if (nq == 0) break;
+    uint8_t *tab = static_cast<uint8_t *>(B.tab[b].p);
+    CU_TRY(cudaMemcpyAsync(tab, B.pinned[b], B.bytes(), cudaMemcpyHostToDevice, s));
+    RunArgs a{};
+    a.nets = reinterpret_cast<const NetDev *>(tab);
+    a.wins = reinterpret_cast<const NetWin *>(tab + B.wins_at());
+    a.tile_pre = reinterpret_cast<const uint32_t *>(tab + B.pre_at());
+    a.bar = reinterpret_cast<uint32_t *>(tab + B.bar_at());
+    a.n_nets = (uint32_t)n;
+    a.n_tiles = n_tiles;
+    a.steps = (uint32_t)std::min<uint64_t>(window, most);
+    a.nd_max = nd_max;
+    a.kmin = hs[0]->L.kmin;
+    // a network that advances: its recording block is copied and checked, and the exchange periods of all that
+    // advance are counted from its first step (one that has stopped keeps the step, and phase, of its end)
+    int first = 0;
+    while (!p.adv[first]) ++first;
+    a.phase = (uint32_t)(p.t0s[first] % a.kmin);
+    a.status = &reinterpret_cast<const NetDev *>(B.pinned[b])[first].rec->status;
+    CU_TRY(launch_run(a, shape, L2Window{}, s));
+    ++hs[0]->launches;
+    hs[0]->h2d += B.bytes();
+    for (int i = 0; i < n; ++i) {
+      t_issue[i] += p.adv[i];
+      left[i] -= p.adv[i];
+    }
+    for (int i = 0; i < n; ++i)
+      if (p.adv[i]) {
+        int rc = drain_copy_block(hs[i], b, p.adv[i], s);
+        if (rc) return rc;
+      }
+    CU_TRY(cudaEventRecord(B.ev_block[b], s));
+    q[nq++] = std::move(p);
+    next_b ^= 1;
+    return SNN_OK;
+  };
+  auto drain = [&]() -> int {
     Pending p = std::move(q[0]);
     q[0] = std::move(q[1]);
     --nq;
-    status = drain_batch(hs, p.b, p.t0s.data(), p.adv.data(), n, B.ev_block[p.b], B.copy_stream, s);
-    if (status == SNN_OK)
-      for (int i = 0; i < n; ++i) hs[i]->t = p.t0s[i] + p.adv[i];
+    int rc = drain_batch(hs, p.b, p.t0s.data(), p.adv.data(), n, B.ev_block[p.b], B.copy_stream, s);
+    if (rc) return rc;
+    for (int i = 0; i < n; ++i) hs[i]->t = p.t0s[i] + p.adv[i];
+    return SNN_OK;
+  };
+  int status = SNN_OK;
+  while (status == SNN_OK) {
+    most = *std::max_element(left.begin(), left.end());
+    if (most > 0 && nq < 2) status = issue();
+    else if (nq > 0) status = drain();
+    else break;
   }
   // nothing left in flight; networks with a stream of their own may use it next
   if (status != SNN_OK || other_streams) cudaStreamSynchronize(s);
+  // networks whose last window was issued but not drained are invalid: a kernel that gave up at a barrier has lost the
+  // state of all of them, and otherwise their device state is ahead of the host's records
+  if (status != SNN_OK) {
+    cudaStreamSynchronize(B.copy_stream);
+    for (int i = 0; i < n; ++i)
+      if (t_issue[i] != hs[i]->t) hs[i]->broken = true;
+  }
   return status;
 }
 

@@ -61,7 +61,8 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess;
 
 // ---- fake kernels
 static uint32_t g_fit = 0xFFFFFFFFu;           // tiles of one launch of the persistent kernel
-static int g_fail_at = -1;                     // its launch that reports a barrier that was not met
+static int g_fail_at = -1;                     // its launch that reports a barrier that was not met,
+static bool g_fail_launch = false;             // or fails itself
 static std::vector<std::vector<std::pair<uint32_t, uint32_t>>> g_runs;   // windows of every launch's networks
 namespace snn {
 int device_sm_count() { return 152; }
@@ -85,8 +86,10 @@ cudaError_t launch_run(const RunArgs &a, const RunShape &, const L2Window &, cud
     // the exchange period is counted from one phase for all networks that advance
     if (x.t_end > x.t0) CHECK(a.phase == x.t0 % a.kmin);
   }
-  if ((int)g_runs.size() == g_fail_at) *a.status |= kStatusBarrier;
+  const int at = (int)g_runs.size();
   g_runs.push_back(w);
+  if (at == g_fail_at && g_fail_launch) return cudaErrorLaunchOutOfResources;
+  if (at == g_fail_at) *a.status |= kStatusBarrier;
   return cudaSuccess;
 }
 }  // namespace snn
@@ -151,8 +154,42 @@ static void check_phase() {
   }
 }
 
+// A launch that fails: of its networks, those whose windows it (or one still in
+// flight) was to advance answer SNN_ERR_STATE from then on; the others go on.
+static void check_failure() {
+  const uint64_t one[1] = {1};
+  for (bool launch : {false, true})
+    for (int at : {0, 1, 2, 3}) {
+      auto hs = networks(4, 20, 1, 10);
+      const std::vector<uint64_t> steps = {15, 200, 0, 200};
+      g_runs.clear();
+      g_fail_at = at;
+      g_fail_launch = launch;
+      CHECK(snn_run_batch(hs.data(), steps.data(), 4) == SNN_ERR_CUDA);
+      g_fail_at = -1;
+      for (int i = 0; i < 4; ++i) {
+        const uint64_t undrained = launch ? (uint64_t)(10 * at) : (uint64_t)(10 * at + 20);   // issued: two in flight
+        const uint64_t drained = launch ? (uint64_t)(10 * std::max(0, at - 1)) : (uint64_t)(10 * at);
+        const bool lost = std::min(steps[i], undrained) > std::min(steps[i], drained);
+        CHECK(hs[i]->t == std::min(steps[i], drained));
+        CHECK(snn_run_batch(&hs[i], one, 1) == (lost ? SNN_ERR_STATE : SNN_OK));
+      }
+      free_all(hs);
+    }
+  // the same of a single network
+  auto hs = networks(1, 20, 1, 10);
+  g_runs.clear();
+  g_fail_at = 1;
+  g_fail_launch = true;
+  CHECK(snn_run(hs[0], 100) == SNN_ERR_CUDA);
+  CHECK(snn_run(hs[0], 1) == SNN_ERR_STATE);
+  free_all(hs);
+  g_fail_at = -1;
+  g_fail_launch = false;
+}
+
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}};
+  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}};
   if (argc != 2 || !checks.count(argv[1])) return 2;
   checks.at(argv[1])();
   std::puts("ok");
