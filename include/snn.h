@@ -168,10 +168,12 @@ int snn_run(snn_handle h, uint64_t steps);
 
 /* Advance n networks together by steps[i] each, in lockstep in one launch of
  * the persistent kernel per window (networks that reach their count stop
- * early; networks of different smallest delays, or more than fit one launch,
- * take turns).  Each network's results are identical to snn_run on it alone.
- * The networks must share one device; the call is ordered on the first
- * network's stream.
+ * early; networks of different smallest delays or phases of it, or more than
+ * fit one launch, take turns; networks too large for a launch follow together,
+ * each on a stream of its own).  Each network's results are identical to
+ * snn_run on it alone.  The networks must share one device; a launch is ordered
+ * on the stream of its first network, behind the others' streams, and ends
+ * before the call returns.
  * Errors as snn_run, plus SNN_ERR_ARG (a network twice or NULL) and
  * SNN_ERR_LIMIT (more than 65535 networks).  The paper has no counterpart:
  * batching independent networks is a systems pattern of this library. */

@@ -946,6 +946,7 @@ struct PlainRunner {
     uint64_t t0, n;
   };
   snn_net *h = nullptr;
+  cudaStream_t stream = nullptr;
   uint32_t window = 0;
   uint64_t steps = 0, issued = 0, t_issue = 0;
   RunShape shape;   // persistent kernel (blocks > 0), else two kernels per step
@@ -987,7 +988,7 @@ static int runner_issue(PlainRunner &r) {
     // the barrier words follow the header in the recording block, which is zero at every window start
     a.bar = reinterpret_cast<uint32_t *>(base + h->L.off_rec[b] + 128);
     a.status = &a.nd.rec->status;
-    CU_TRY(launch_run(a, r.shape, r.l2, h->stream));
+    CU_TRY(launch_run(a, r.shape, r.l2, r.stream));
     ++h->launches;
   } else {
     NetWin *pw = h->pinned_win + b;   // free: the copy of its last use finished before that drain
@@ -996,14 +997,14 @@ static int runner_issue(PlainRunner &r) {
     uint32_t kernels = 0;
     rc = window_graph(h, b, (uint32_t)(t0 % h->L.nbuf), &gx, &kernels);
     if (rc) return rc;
-    CU_TRY(cudaMemcpyAsync(base + h->L.off_win[b], pw, sizeof(NetWin), cudaMemcpyHostToDevice, h->stream));
-    CU_TRY(cudaGraphLaunch(gx, h->stream));
+    CU_TRY(cudaMemcpyAsync(base + h->L.off_win[b], pw, sizeof(NetWin), cudaMemcpyHostToDevice, r.stream));
+    CU_TRY(cudaGraphLaunch(gx, r.stream));
     h->h2d += sizeof(NetWin);
     h->launches += kernels;
   }
   r.issued += n;
   r.t_issue += n;
-  rc = drain_copy_block(h, b, n, h->stream);
+  rc = drain_copy_block(h, b, n, r.stream);
   if (rc) return rc;
   r.q[r.nq++] = PlainRunner::Pending{b, t0, n};
   r.next_b ^= 1;
@@ -1014,13 +1015,14 @@ static int runner_drain(PlainRunner &r) {
   const PlainRunner::Pending p = r.q[0];
   r.q[0] = r.q[1];
   --r.nq;
-  int rc = drain_finish(r.h, p.b, p.t0, r.h->stream);
+  int rc = drain_finish(r.h, p.b, p.t0, r.stream);
   if (rc == SNN_OK) r.h->t = p.t0 + p.n;
   return rc;
 }
 
 static int runner_start(PlainRunner &r, snn_net *h, uint64_t steps) {
   r.h = h;
+  r.stream = h->stream;
   r.window = plain_window(h);
   r.steps = steps;
   r.t_issue = h->t;
@@ -1033,7 +1035,7 @@ static int runner_start(PlainRunner &r, snn_net *h, uint64_t steps) {
 // issued but not drained is invalid (its device state is ahead of the host's
 // records, or lost with the kernel).
 static void runner_failed(PlainRunner &r) {
-  cudaStreamSynchronize(r.h->stream);
+  cudaStreamSynchronize(r.stream);
   if (r.t_issue != r.h->t) r.h->broken = true;
 }
 
@@ -1047,15 +1049,22 @@ static int run_plain(snn_net *h, uint64_t steps) {
   return status;
 }
 
-// Several networks on the two-kernel path, each on its own stream: their
-// windows are issued and drained round robin from this thread, so the kernels
-// of different networks overlap on the GPU.
-static int run_plain_many(snn_net *const *hs, const uint64_t *steps, int32_t n) {
+// Several networks, each on its own stream: their windows are issued and
+// drained round robin from this thread, so the kernels of different networks
+// overlap on the GPU.  With `split`, networks that share a stream are spread
+// over private ones, ordered behind it and finished when the call returns.
+static int run_plain_many(snn_net *const *hs, const uint64_t *steps, int32_t n, bool split) {
   std::vector<PlainRunner> rs((size_t)n);
   for (int i = 0; i < n; ++i) {
     int rc = runner_start(rs[i], hs[i], steps[i]);
     if (rc) return rc;
   }
+  for (int i = 1; split && i < n; ++i)
+    if (std::any_of(hs, hs + i, [&](const snn_net *h) { return h->stream == hs[i]->stream; })) {
+      CU_TRY(cudaEventRecord(hs[i]->ev_block[0], hs[i]->stream));   // the last window's reset may still be on its way
+      CU_TRY(cudaStreamWaitEvent(hs[i]->cap_stream, hs[i]->ev_block[0], 0));
+      rs[i].stream = hs[i]->cap_stream;
+    }
   int status = SNN_OK;
   bool any = true;
   while (status == SNN_OK && any) {
@@ -1068,6 +1077,8 @@ static int run_plain_many(snn_net *const *hs, const uint64_t *steps, int32_t n) 
   }
   if (status != SNN_OK)
     for (auto &r : rs) runner_failed(r);
+  for (int i = 0; i < n; ++i)
+    if (rs[i].stream != hs[i]->stream) cudaStreamSynchronize(rs[i].stream);
   return status;
 }
 
@@ -1237,34 +1248,46 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
 }
 
 // A set of networks: grouped by smallest delay and phase, each group in as few
-// launches side by side as the blocks' shared memory allows.
+// launches side by side as the blocks' shared memory allows.  Networks too large
+// for a launch take two kernels per step, on streams of their own: one after the
+// other they leave the GPU idle between their kernels (us a step of all, in turns
+// and so: eight of 12x12 modules with smallest delay 50 69 and 32, four of 8x8
+// with 100 32 and 15, two of 24x24 with 10 29 and 22).
 static int run_set(snn_net *const *hs, const uint64_t *steps, int32_t n) {
-  std::vector<int32_t> order(n);
-  for (int32_t i = 0; i < n; ++i) order[i] = i;
-  auto key = [&](int32_t i) { return std::make_pair(hs[i]->L.kmin, hs[i]->t % hs[i]->L.kmin); };
-  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return key(x) < key(y); });
+  std::vector<int32_t> order;
+  std::vector<snn_net *> big;
+  std::vector<uint64_t> big_steps;
   const snn_launch &cfg = hs[0]->cfg;
   const int threads = cfg.path == 1 ? std::min(1024, cfg.fused_block * cfg.fused_items_per_sm) : 1024;
-  for (int32_t at = 0; at < n;) {
+  for (int32_t i = 0; i < n; ++i) {
+    if (run_shape(hs[i]->L.N_pad / 128u, hs[i]->L.kmin, threads, 1u).blocks > 0) {
+      order.push_back(i);
+    } else {
+      big.push_back(hs[i]);
+      big_steps.push_back(steps[i]);
+    }
+  }
+  auto key = [&](int32_t i) { return std::make_pair(hs[i]->L.kmin, hs[i]->t % hs[i]->L.kmin); };
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return key(x) < key(y); });
+  for (size_t at = 0; at < order.size();) {
     std::vector<snn_net *> g;
     std::vector<uint64_t> st;
     RunShape shape;
     uint64_t tiles = 0;
-    while (at < n && (g.empty() || key(order[at]) == std::make_pair(g[0]->L.kmin, g[0]->t % g[0]->L.kmin))) {
+    while (at < order.size() && (g.empty() || key(order[at]) == std::make_pair(g[0]->L.kmin, g[0]->t % g[0]->L.kmin))) {
       snn_net *h = hs[order[at]];
       const RunShape next = run_shape((uint32_t)(tiles + h->L.N_pad / 128u), h->L.kmin, threads, (uint32_t)g.size() + 1u);
-      if (next.blocks < 1 && !g.empty()) break;
+      if (next.blocks < 1) break;
       g.push_back(h);
       st.push_back(steps[order[at]]);
       tiles += h->L.N_pad / 128u;
       shape = next;
       ++at;
-      if (next.blocks < 1) break;   // too large for the persistent kernel by itself
     }
     const int rc = g.size() == 1 ? run_plain(g[0], st[0]) : run_lockstep(g.data(), st.data(), (int32_t)g.size(), shape, (uint32_t)tiles);
     if (rc) return rc;
   }
-  return SNN_OK;
+  return big.empty() ? SNN_OK : run_plain_many(big.data(), big_steps.data(), (int32_t)big.size(), true);
 }
 
 // Two large networks that leave the form to the library run as two kernels per
@@ -1290,7 +1313,7 @@ static bool run_apart(snn_net *const *hs, const uint64_t *steps, int32_t n) {
 static int run_together(snn_net *const *hs, const uint64_t *steps, int32_t n) {
   bool together = n > 1;
   for (int i = 0; i < n; ++i) together &= has_default_shape(hs[i]->cfg);
-  if (!together) return run_plain_many(hs, steps, n);
+  if (!together) return run_plain_many(hs, steps, n, false);
   if (!run_apart(hs, steps, n)) return run_set(hs, steps, n);
   struct Shapes {   // for this call only
     snn_net *const *hs;
@@ -1309,7 +1332,7 @@ static int run_together(snn_net *const *hs, const uint64_t *steps, int32_t n) {
       for (int i = 0; i < 2; ++i) hs[i]->cfg = kept[i];
     }
   } shapes(hs);
-  return run_plain_many(hs, steps, n);
+  return run_plain_many(hs, steps, n, false);
 }
 
 // ---------------------------------------------------------------------------

@@ -17,6 +17,7 @@
   } while (0)
 
 // ---- fake CUDA runtime
+static std::vector<cudaStream_t> g_graph_streams;   // of every graph launched
 static uintptr_t g_next_id = 16;
 template <class T>
 static cudaError_t new_handle(T *out) {
@@ -56,7 +57,7 @@ cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventRecordWithFlags(cudaEvent_t, cudaStream_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 1.0f; return cudaSuccess; }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t s) { g_graph_streams.push_back(s); return cudaSuccess; }
 }
 
 // ---- fake kernels
@@ -188,8 +189,29 @@ static void check_failure() {
   g_fail_launch = false;
 }
 
+// Networks too large for a launch of the persistent kernel advance side by side
+// on streams of their own, also when the caller gave them one stream.
+static void check_large() {
+  g_fit = 12;   // a network of one module has 10 tiles, one of two 20
+  for (bool one_stream : {false, true}) {
+    std::vector<snn_handle> hs;
+    for (int gx : {2, 1, 2, 2}) hs.push_back(networks(1, 20, 3, 10, gx)[0]);
+    for (size_t i = 0; i < hs.size(); ++i) hs[i]->stream = reinterpret_cast<cudaStream_t>(uintptr_t(one_stream ? 1 : i + 1));
+    const std::vector<uint64_t> steps = {25, 25, 0, 40};
+    g_runs.clear();
+    g_graph_streams.clear();
+    CHECK(snn_run_batch(hs.data(), steps.data(), 4) == SNN_OK);
+    for (size_t i = 0; i < hs.size(); ++i) CHECK(hs[i]->t == steps[i]);
+    CHECK(g_runs.size() == 3 && g_graph_streams.size() == 3 + 4);
+    // the second network's first window is launched before the first network's third
+    std::set<cudaStream_t> first(g_graph_streams.begin(), g_graph_streams.begin() + 4);
+    CHECK(first.size() == 2);
+    free_all(hs);
+  }
+}
+
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}};
+  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}, {"large", check_large}};
   if (argc != 2 || !checks.count(argv[1])) return 2;
   checks.at(argv[1])();
   std::puts("ok");

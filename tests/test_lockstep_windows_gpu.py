@@ -50,3 +50,23 @@ def test_server_with_exchange_periods():
         assert len(st) and np.array_equal(out[i].spike_steps, st) and np.array_equal(out[i].spike_ids, ids)
         assert np.array_equal(out[i].rates, g.rates())
         g.close()
+
+
+def test_networks_beyond_one_launch(oracle_mod):
+    """Two networks too large for the persistent kernel and a small one, all on
+    one stream: the large ones advance side by side on streams of their own."""
+    import paper_1902_08410_gb300 as snn
+    nets, params = [], []
+    for i, (gx, gy) in enumerate(((44, 44), (2, 2), (45, 43))):
+        p = W.base_params(gx, gy, 1.0, "AW", record_format=i % 2)
+        p.update(out_degree=9, V_th=[10.0] * 3, V_r=[0.0] * 3)   # active with few synapses
+        params.append(p)
+        nets.append(snn.Network(p, 70 + i))
+        nets[i].launch = {"window_steps": 8}
+    for run, steps in (("run_batch", (19, 21, 10)), ("run_concurrent", (7, 3, 12))):
+        getattr(snn, run)(nets, steps)
+    for i, (g, n) in enumerate(zip(nets, (26, 24, 22))):
+        o = oracle_mod.OracleNet(params[i], 70 + i)
+        o.run(n)
+        assert_same(gpu_results(g), oracle_results(o), n)
+        g.close()
