@@ -872,18 +872,30 @@ static int drain_absorb(snn_net *h, int b, uint64_t t0, uint32_t n_rec, cudaStre
   const unsigned long long *ext = reinterpret_cast<const unsigned long long *>(blk + (L.off_ext[b] - L.off_rec[b]));
   for (uint32_t i = 0; i < L.n_ext_slots; ++i) h->ext_events += ext[i];
   if (n_rec) {
-    // blocks record a step's spikes after they have met the others, so entries of neighbouring steps (of a whole
-    // exchange period) may come mixed: grouped by step here, the order within a step is left to the readers
+    // The update kernel leaves entries in the order of the steps, and they are taken as they come.  Blocks of the
+    // persistent kernel record a step's spikes after they have met the others, so entries of neighbouring steps (of a
+    // whole exchange period) may come mixed, and are grouped by step; the order within a step is left to the readers.  Grouping every window cost 2 ns an entry: a call of 60 steps of 2.42M
+    // neurons, which has one window and nothing to hide it behind, took 6.7 ms with 510k spikes, 5.1 so.
     const size_t old = h->raster.size();
     h->raster.resize(old + n_rec);
-    std::vector<uint32_t> at(L.window + 1u, 0u);
-    for (uint32_t i = 0; i < n_rec; ++i) ++at[((h->entries[i] >> 32) & 0xFFFFu) + 1u];
-    for (uint32_t k = 0; k < L.window; ++k) at[k + 1u] += at[k];
     unsigned long long *to = h->raster.data() + old;
-    for (uint32_t i = 0; i < n_rec; ++i) {
-      const unsigned long long e = h->entries[i];
-      const uint64_t k = (e >> 32) & 0xFFFFu;
-      to[at[k]++] = ((t0 + k) << 32) | (e & 0xFFFFFFFFull);
+    auto step_of = [&](uint32_t i) { return (uint32_t)(h->entries[i] >> 32) & 0xFFFFu; };
+    auto entry = [&](uint32_t i, uint32_t k) { return ((t0 + k) << 32) | (h->entries[i] & 0xFFFFFFFFull); };
+    uint32_t from = 0;
+    for (uint32_t last = 0; from < n_rec; ++from) {
+      const uint32_t k = step_of(from);
+      if (k < last) break;
+      to[from] = entry(from, k);
+      last = k;
+    }
+    if (from < n_rec) {
+      std::vector<uint32_t> at(L.window + 1u, 0u);
+      for (uint32_t i = 0; i < n_rec; ++i) ++at[step_of(i) + 1u];
+      for (uint32_t k = 0; k < L.window; ++k) at[k + 1u] += at[k];
+      for (uint32_t i = 0; i < n_rec; ++i) {
+        const uint32_t k = step_of(i);
+        to[at[k]++] = entry(i, k);
+      }
     }
   }
   // rates of the window, bins from t0 / bin_steps
