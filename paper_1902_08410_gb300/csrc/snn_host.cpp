@@ -972,7 +972,7 @@ struct PlainRunner {
 static RunShape plain_shape(const snn_net *h) {
   if (h->cfg.path == 0 && !has_default_shape(h->cfg)) return RunShape{};
   const int threads = h->cfg.path == 1 ? h->cfg.fused_block * h->cfg.fused_items_per_sm : 1024;
-  return run_shape(h->L.N_pad / 128u, h->L.kmin, std::min(threads, 1024), 1u);
+  return run_shape(h->L.N_pad / 128u, h->L.kmin, std::min(threads, 1024), 1u, false);
 }
 
 static uint32_t plain_window(const snn_net *h) {
@@ -1260,44 +1260,67 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
 }
 
 // A set of networks: grouped by smallest delay and phase, each group in as few
-// launches side by side as the blocks' shared memory allows.  Networks too large
-// for a launch take two kernels per step, on streams of their own: one after the
-// other they leave the GPU idle between their kernels (us a step of all, in turns
-// and so: eight of 12x12 modules with smallest delay 50 69 and 32, four of 8x8
-// with 100 32 and 15, two of 24x24 with 10 29 and 22).
-static int run_set(snn_net *const *hs, const uint64_t *steps, int32_t n) {
-  std::vector<int32_t> order;
-  std::vector<snn_net *> big;
-  std::vector<uint64_t> big_steps;
-  const snn_launch &cfg = hs[0]->cfg;
-  const int threads = cfg.path == 1 ? std::min(1024, cfg.fused_block * cfg.fused_items_per_sm) : 1024;
-  for (int32_t i = 0; i < n; ++i) {
-    if (run_shape(hs[i]->L.N_pad / 128u, hs[i]->L.kmin, threads, 1u).blocks > 0) {
-      order.push_back(i);
-    } else {
-      big.push_back(hs[i]);
-      big_steps.push_back(steps[i]);
+// launches side by side as the blocks' shared memory allows.
+struct Member {
+  snn_net *h;
+  uint64_t steps;
+};
+
+// The launches of `ms`; `part` as for run_shape.  Networks too large for a launch,
+// and with `part` those that would be alone in one, are left in `ms`.
+static int run_groups(std::vector<Member> &ms, int threads, bool part) {
+  auto key = [](const Member &m) { return std::make_pair(m.h->L.kmin, m.h->t % m.h->L.kmin); };
+  auto tiles = [](const Member &m) { return m.h->L.N_pad / 128u; };
+  std::vector<Member> left;
+  std::stable_sort(ms.begin(), ms.end(), [&](const Member &x, const Member &y) { return key(x) < key(y); });
+  for (size_t at = 0; at < ms.size();) {
+    const size_t from = at;
+    RunShape shape;
+    uint64_t n_tiles = 0;
+    for (; at < ms.size() && key(ms[at]) == key(ms[from]); ++at) {
+      const RunShape next = run_shape((uint32_t)(n_tiles + tiles(ms[at])), ms[at].h->L.kmin, threads, (uint32_t)(at - from) + 1u, part);
+      if (next.blocks < 1) break;
+      n_tiles += tiles(ms[at]);
+      shape = next;
     }
-  }
-  auto key = [&](int32_t i) { return std::make_pair(hs[i]->L.kmin, hs[i]->t % hs[i]->L.kmin); };
-  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return key(x) < key(y); });
-  for (size_t at = 0; at < order.size();) {
+    const size_t n = at - from;
+    if (n == 0 || (part && n == 1)) {
+      left.push_back(ms[from]);
+      at = from + 1;
+      continue;
+    }
     std::vector<snn_net *> g;
     std::vector<uint64_t> st;
-    RunShape shape;
-    uint64_t tiles = 0;
-    while (at < order.size() && (g.empty() || key(order[at]) == std::make_pair(g[0]->L.kmin, g[0]->t % g[0]->L.kmin))) {
-      snn_net *h = hs[order[at]];
-      const RunShape next = run_shape((uint32_t)(tiles + h->L.N_pad / 128u), h->L.kmin, threads, (uint32_t)g.size() + 1u);
-      if (next.blocks < 1) break;
-      g.push_back(h);
-      st.push_back(steps[order[at]]);
-      tiles += h->L.N_pad / 128u;
-      shape = next;
-      ++at;
+    for (size_t i = from; i < at; ++i) {
+      g.push_back(ms[i].h);
+      st.push_back(ms[i].steps);
     }
-    const int rc = g.size() == 1 ? run_plain(g[0], st[0]) : run_lockstep(g.data(), st.data(), (int32_t)g.size(), shape, (uint32_t)tiles);
+    const int rc = n == 1 ? run_plain(g[0], st[0]) : run_lockstep(g.data(), st.data(), (int32_t)n, shape, (uint32_t)n_tiles);
     if (rc) return rc;
+  }
+  ms = std::move(left);
+  return SNN_OK;
+}
+
+// What does not fit a launch with the drives of a whole exchange period may fit
+// with part of them.  Networks too large for that too take two kernels per step,
+// on streams of their own: one after the other they leave the GPU idle between
+// their kernels (us a step of all, in turns and so: two of 24x24 modules with
+// smallest delay 10 29 and 22).
+static int run_set(snn_net *const *hs, const uint64_t *steps, int32_t n) {
+  const snn_launch &cfg = hs[0]->cfg;
+  const int threads = cfg.path == 1 ? std::min(1024, cfg.fused_block * cfg.fused_items_per_sm) : 1024;
+  std::vector<Member> ms;
+  for (int32_t i = 0; i < n; ++i) ms.push_back(Member{hs[i], steps[i]});
+  for (bool part : {false, true}) {
+    const int rc = run_groups(ms, threads, part);
+    if (rc) return rc;
+  }
+  std::vector<snn_net *> big;
+  std::vector<uint64_t> big_steps;
+  for (const Member &m : ms) {
+    big.push_back(m.h);
+    big_steps.push_back(m.steps);
   }
   return big.empty() ? SNN_OK : run_plain_many(big.data(), big_steps.data(), (int32_t)big.size(), true);
 }

@@ -151,7 +151,7 @@ struct RunArgs {
   uint32_t visit;             // steps between two visits of a live spike (1 in the period form)
   uint32_t fifo;              // live spikes of one ring that a block holds in shared memory (power of two)
   uint32_t nt;                // tiles of a block, at most
-  uint32_t drives;            // external drives kept per neuron: kmin in the period form, else 1 or 2
+  uint32_t drives;            // external drives kept per neuron: kmin or less in the period form, else 1 or 2
   uint32_t pre;               // records of a new spike's row prefetched (multiple of 8)
   // {grid barrier count, last step (+1) that overflowed a live list, lists not taken over}, zero at launch
   uint32_t *bar;
@@ -164,8 +164,8 @@ struct RunShape {
   uint32_t tables = 0;        // networks whose descriptors fit in shared memory beside the rest
   size_t smem = 0;
 };
-// blocks == 0: too many tiles for one launch.
-RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_nets);
+// blocks == 0: too many tiles for one launch.  `part`: the drives of part of an exchange period will do.
+RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_nets, bool part);
 cudaError_t launch_run(const RunArgs &a, const RunShape &sh, const L2Window &l2, cudaStream_t s);
 cudaError_t prepare_run_kernels();
 // Delivery keeps each warp's segment prefix in registers, in chunks of 32

@@ -112,8 +112,10 @@ __device__ __forceinline__ bool pass_after(const NetDev &nd, uint32_t t) { retur
 //            visit + 2 input buffers rotate: step k uses buffer k mod (visit +
 //            2), cleared by its update, and is next added to from step k + 1 on,
 //            after the barrier that ends step k.
-//   kPeriod  kmin > 1.  The grid meets once per exchange period of kmin steps;
-//            all live spikes are visited before it.  2 kmin input buffers: the
+//   kPeriod  kmin > 1.  The grid meets once per exchange period of kmin steps
+//            (where only the drives of part of a period fit, after each part);
+//            all live spikes are visited before the meeting that ends a period.
+//            2 kmin input buffers: the
 //            updates of a period read and clear its own, the pass after it adds
 //            into those of the next kmin steps.
 enum RunForm { kAhead, kPeriod };
@@ -516,7 +518,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
   };
   const uint32_t phase0 = PERIOD ? a.phase : 0u;
   auto interval = [&](uint32_t k) {   // steps until the grid meets again
-    return PERIOD ? min(a.kmin - (phase0 + k) % a.kmin, a.steps - k) : 1u;
+    return PERIOD ? min(min(a.kmin - (phase0 + k) % a.kmin, P), a.steps - k) : 1u;
   };
   __syncthreads();
   draw(0u, interval(0u), (met & 1u) ^ 1u, s.pend[0]);
@@ -815,7 +817,14 @@ cudaError_t prepare_run_kernels() {
 // neuron stay in shared memory (2.1M neurons at kmin = 1); what does not fit
 // takes two kernels per step (64x64 modules: 80 us a step, against 125 and 217 us
 // in two forms of this kernel with the state in global memory).
-RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_nets) {
+// `part`: a set that has too many drives for its whole exchange period keeps
+// those of up to 16 steps and 1024 live spikes at least, and the grid meets
+// within the period.  us a step of all networks, as two kernels side by side and
+// so: four of 8x8 modules with smallest delay 100 15.6 and 3.2, eight of 4x4 with
+// 254 24 and 2.4, six of 16x16 with 100 25 and 16.  Room for four steps' drives is
+// the line: two of 22x22 with 20 (five) 17.1 and 16.0, two of 20x20 (six) 16.1 and
+// 16.1, but two of 24x24 with 10 (three) 20.6 and 28, two of 28x28 (two) 25 and 33.
+RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_nets, bool part) {
   RunShape sh;
   const uint32_t sms = (uint32_t)std::max(1, device_sm_count());
   sh.blocks = (int)std::max(1u, std::min(sms, n_tiles));
@@ -829,6 +838,11 @@ RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_
   // Drives a step further ahead where they fit: the neurons with several external events are then completed beside
   // the visits instead of behind a block barrier.
   sh.drives = sh.form == kPeriod ? kmin : (run_smem(2u, sh.nt, sh.visit * sh.fifo) <= budget ? 2u : 1u);
+  if (part && sh.form == kPeriod && run_smem(kmin, sh.nt, sh.fifo) > budget) {
+    sh.fifo = 1024u;
+    sh.drives = std::min(kmin, 16u);
+    while (sh.drives > 4u && run_smem(sh.drives, sh.nt, sh.fifo) > budget) --sh.drives;
+  }
   const size_t tables = n_nets > 1u ? n_nets * (sizeof(NetDev) + sizeof(NetWin)) : 0u;
   sh.tables = tables && run_smem(sh.drives, sh.nt, sh.visit * sh.fifo) + tables <= budget ? n_nets : 0u;
   const size_t fixed = sh.tables ? tables : 0u;

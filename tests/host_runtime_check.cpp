@@ -73,7 +73,7 @@ cudaError_t launch_build_rows(const NetDev &, const BuildDev &, cudaStream_t) { 
 cudaError_t launch_init_state(const NetDev &, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_update(const NetDev &, uint32_t, StepMod, int, int, const L2Window &, bool, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_deliver(const NetDev &, uint32_t, StepMod, uint32_t, int, int, const L2Window &, bool, cudaStream_t) { return cudaSuccess; }
-RunShape run_shape(uint32_t n_tiles, uint32_t, int threads, uint32_t) {
+RunShape run_shape(uint32_t n_tiles, uint32_t, int threads, uint32_t, bool) {
   RunShape s;
   s.blocks = n_tiles <= g_fit ? 1 : 0;
   s.threads = threads;

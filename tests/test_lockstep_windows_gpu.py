@@ -70,3 +70,35 @@ def test_networks_beyond_one_launch(oracle_mod):
         o.run(n)
         assert_same(gpu_results(g), oracle_results(o), n)
         g.close()
+
+
+@pytest.mark.parametrize("grids,n_delay,min_delay,volley,calls", [
+    (((4, 4), (5, 4), (4, 4)), 254, 254, False, [(600, 333, 0), (45, 1300, 777)]),
+    (((8, 8), (8, 9)), 120, 100, False, [(150, 130), (7, 95)]),
+    (((16, 16), (16, 15)), 33, 30, True, [(22, 35), (41, 9)])])
+def test_part_of_an_exchange_period(oracle_mod, grids, n_delay, min_delay, volley, calls):
+    """Sets whose networks do not fit a launch with the drives of a whole
+    exchange period: the grid meets within the period too.  Networks that stop
+    at any step, in the second call networks of different phases, and more live
+    spikes than the lists hold."""
+    import paper_1902_08410_gb300 as snn
+    nets, params = [], []
+    for i, (gx, gy) in enumerate(grids):
+        p = W.base_params(gx, gy, 1.0, "AW", record_format=i % 2)
+        p.update(out_degree=9 if volley else 40, n_delay=n_delay, min_delay=min_delay)
+        p.update(V_th=[1.0] * 3 if volley else [10.0] * 3, V_r=[0.0] * 3)
+        if volley:
+            p["tau_arp"] = [0.3, 0.2, 0.1]
+        params.append(p)
+        nets.append(snn.Network(p, 30 + i))
+    for j, steps in enumerate(calls):
+        before = sum(g.stats()["kernel_launches"] for g in nets)
+        snn.run_batch(nets, steps)
+        if j == 0:   # in one phase: a launch per window, not per step
+            assert sum(g.stats()["kernel_launches"] for g in nets) - before <= 4
+    for i, g in enumerate(nets):
+        n = sum(c[i] for c in calls)
+        o = oracle_mod.OracleNet(params[i], 30 + i)
+        o.run(n)
+        assert_same(gpu_results(g), oracle_results(o), n)
+        g.close()
