@@ -142,7 +142,8 @@ int snn_set_allocator(snn_alloc_fn alloc, snn_free_fn free_fn, void *ctx);
 
 /* Device bytes a network with these parameters will hold once built
  * (synapse records and their delay-group table, neuron state, 2 max(1, min_delay)
- * input buffers and 4 more for the persistent kernel, spike history of the last
+ * input buffers, 4 more for grids that the persistent kernel can take (it uses
+ * them with a smallest delay of 1), spike history of the last
  * n_delay + max(1, min_delay) steps, tables, recording buffers). */
 int snn_footprint(const snn_params *p, size_t *bytes_out);
 

@@ -260,8 +260,8 @@ void build_inputs(const snn_params &p, BuildDev &bd) {
 // ---------------------------------------------------------------------------
 // Device arena of one network, in this order: V, c, ref, the spike counts of the
 // last n_delay + min_delay steps, 2 min_delay input buffers, the spike lists
-// (everything a run leaves behind), the persistent kernel's further input
-// buffers (zero between windows), synapse rows, their delay-group table, amplitude table, two windows, two recording blocks
+// (everything a run leaves behind), the further input buffers of the persistent
+// kernel with a smallest delay of 1 (zero between windows), synapse rows, their delay-group table, amplitude table, two windows, two recording blocks
 // (header, external-event slots, rate window: one contiguous copy per window),
 // two raster entry buffers.  Windows alternate between the two buffer sets, so
 // the host drains one window's records while the GPU runs the next.
@@ -339,7 +339,7 @@ static Layout make_layout(const snn_params &p) {
   L.off_cnt = take((size_t)L.D * 4);
   L.off_acc = take((size_t)L.nbuf * L.N_pad * 4);
   L.off_hist = take((size_t)L.D * L.N_pad * 4);   // right behind acc: N_pad * 4 is a multiple of 256
-  L.off_more = take((size_t)kMaxVisit * L.N_pad * 4);
+  L.off_more = take(L.N_pad / 128u <= kRunMaxTiles ? (size_t)kMaxVisit * L.N_pad * 4 : 0u);
   L.off_rows = take((size_t)L.N * L.row_bytes);
   L.off_offs = take((size_t)L.N * L.os * 2);
   L.off_amp = take((size_t)kNPop * kZTab * 4);
@@ -699,7 +699,7 @@ extern "C" int snn_build_network(const snn_params *p, uint64_t seed, void *cuda_
   bd.cdf = d_cdf;
   bd.ztab = d_z;
   CU_TRY(cudaMemsetAsync(base + L.off_cnt, 0, L.off_hist - L.off_cnt, s));   // spike counts, inputs
-  CU_TRY(cudaMemsetAsync(base + L.off_more, 0, L.off_rows - L.off_more, s));
+  if (L.off_rows > L.off_more) CU_TRY(cudaMemsetAsync(base + L.off_more, 0, L.off_rows - L.off_more, s));
   CU_TRY(cudaMemsetAsync(base + L.off_win[0], 0, L.off_entries[0] - L.off_win[0], s));   // windows, blocks
   CU_TRY(cudaMallocHost(&h->pinned_win, 2 * sizeof(NetWin)));
   std::memset(h->pinned_win, 0, 2 * sizeof(NetWin));

@@ -133,6 +133,10 @@ cudaError_t launch_deliver(const NetDev &nd, uint32_t k, StepMod km, uint32_t la
 // Persistent kernel: steps between two visits of a live spike, at most; kmin = 1
 // networks have visit + 2 input buffers.
 constexpr uint32_t kMaxVisit = 4;
+// Tiles of one launch at most: a block's shared memory holds the state of fewer
+// than 128, on 152 SMs.  Grids above hold no further input buffers (64x64 modules:
+// 82 MB); a constant, so that snn_footprint needs no device.
+constexpr uint32_t kRunMaxTiles = 128u * 152u;
 
 // Persistent kernel: a window of steps of one or more networks in one launch
 // (snn_run.cu).

@@ -849,7 +849,7 @@ RunShape run_shape(uint32_t n_tiles, uint32_t kmin, int max_threads, uint32_t n_
   while (sh.fifo < 8192u / sh.visit && run_smem(sh.drives, sh.nt, sh.visit * sh.fifo * 2u) + fixed <= budget)
     sh.fifo *= 2u;
   sh.smem = run_smem(sh.drives, sh.nt, sh.visit * sh.fifo) + fixed;
-  if (sh.smem > budget) sh.blocks = 0;   // too many tiles per block
+  if (sh.smem > budget || n_tiles > kRunMaxTiles) sh.blocks = 0;   // too many tiles per block, or in all
   return sh;
 }
 

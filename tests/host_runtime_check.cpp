@@ -210,8 +210,18 @@ static void check_large() {
   }
 }
 
+// Only grids that the persistent kernel can take hold its further input buffers.
+static void check_footprint() {
+  for (int kmin : {1, 4})
+    for (int gx : {2, 1900, 2000}) {   // 2.375M and 2.5M neurons, around 128 tiles on each of 152 SMs
+      const Layout L = make_layout(params(gx, 20, kmin));
+      CHECK(L.off_rows - L.off_more == (gx < 2000 ? (size_t)kMaxVisit * L.N_pad * 4 : 0u));
+      CHECK(L.off_more == L.off_hist + (size_t)L.D * L.N_pad * 4);
+    }
+}
+
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}, {"large", check_large}};
+  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}, {"large", check_large}, {"footprint", check_footprint}};
   if (argc != 2 || !checks.count(argv[1])) return 2;
   checks.at(argv[1])();
   std::puts("ok");
