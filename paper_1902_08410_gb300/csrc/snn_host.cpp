@@ -1099,15 +1099,16 @@ static int run_plain_many(snn_net *const *hs, const uint64_t *steps, int32_t n, 
 // ---------------------------------------------------------------------------
 // Device tables of a batch, one set per calling thread (grown as needed, freed with the thread).
 struct BatchCtx {
-  DevBuf tab[2];               // per buffer set: NetDev[cap], NetWin[cap], tile_pre[cap + 1], barrier words
+  DevBuf tab[2];               // per buffer set, a table of up to `cap` networks
   size_t cap = 0;
   uint8_t *pinned[2] = {nullptr, nullptr};
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_block[2] = {nullptr, nullptr};
-  size_t wins_at() const { return cap * sizeof(NetDev); }
-  size_t pre_at() const { return wins_at() + cap * sizeof(NetWin); }
-  size_t bar_at() const { return align_up(pre_at() + (cap + 1) * 4, 256); }
-  size_t bytes() const { return bar_at() + 256; }
+  // table of n networks: NetDev[n], NetWin[n], tile_pre[n + 1], barrier words
+  static size_t wins_at(size_t n) { return n * sizeof(NetDev); }
+  static size_t pre_at(size_t n) { return wins_at(n) + n * sizeof(NetWin); }
+  static size_t bar_at(size_t n) { return align_up(pre_at(n) + (n + 1) * 4, 256); }
+  static size_t bytes(size_t n) { return bar_at(n) + 256; }
   void drop() {
     for (int b = 0; b < 2; ++b) {
       tab[b].release();
@@ -1144,8 +1145,8 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
     B.drop();
     B.cap = cap;
     for (int b = 0; b < 2; ++b) {
-      int rc = dev_alloc(B.tab[b], B.bytes());
-      cudaError_t e = rc ? cudaSuccess : cudaMallocHost(&B.pinned[b], B.bytes());
+      int rc = dev_alloc(B.tab[b], B.bytes(cap));
+      cudaError_t e = rc ? cudaSuccess : cudaMallocHost(&B.pinned[b], B.bytes(cap));
       if (rc || e != cudaSuccess) {
         B.drop();
         return rc ? rc : fail(SNN_ERR_OOM, std::string("cudaMallocHost: ") + cudaGetErrorString(e));
@@ -1164,7 +1165,7 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
       CU_TRY(cudaStreamSynchronize(hs[i]->stream));
     }
   for (int b = 0; b < 2; ++b) {
-    uint32_t *pre = reinterpret_cast<uint32_t *>(B.pinned[b] + B.pre_at());
+    uint32_t *pre = reinterpret_cast<uint32_t *>(B.pinned[b] + B.pre_at(n));
     pre[0] = 0;
     for (int i = 0; i < n; ++i) {
       NetDev d = descriptor(hs[i], b);
@@ -1172,7 +1173,7 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
       reinterpret_cast<NetDev *>(B.pinned[b])[i] = d;
       pre[i + 1] = pre[i] + hs[i]->L.N_pad / 128u;
     }
-    std::memset(B.pinned[b] + B.bar_at(), 0, 256);
+    std::memset(B.pinned[b] + B.bar_at(n), 0, 256);
   }
 
   // windows alternate between the two buffer sets, two in flight at most
@@ -1187,7 +1188,7 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
   uint64_t most = 0;   // steps left of the network that has most
   auto issue = [&]() -> int {
     const int b = next_b;
-    NetWin *pw = reinterpret_cast<NetWin *>(B.pinned[b] + B.wins_at());   // free: its window has been drained
+    NetWin *pw = reinterpret_cast<NetWin *>(B.pinned[b] + B.wins_at(n));   // free: its window has been drained
     Pending p{b, std::vector<uint64_t>(n), std::vector<uint64_t>(n)};
     for (int i = 0; i < n; ++i) {
       const uint64_t adv = std::min<uint64_t>(window, left[i]);
@@ -1197,12 +1198,12 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
       p.adv[i] = adv;
     }
     uint8_t *tab = static_cast<uint8_t *>(B.tab[b].p);
-    CU_TRY(cudaMemcpyAsync(tab, B.pinned[b], B.bytes(), cudaMemcpyHostToDevice, s));
+    CU_TRY(cudaMemcpyAsync(tab, B.pinned[b], B.bytes(n), cudaMemcpyHostToDevice, s));
     RunArgs a{};
     a.nets = reinterpret_cast<const NetDev *>(tab);
-    a.wins = reinterpret_cast<const NetWin *>(tab + B.wins_at());
-    a.tile_pre = reinterpret_cast<const uint32_t *>(tab + B.pre_at());
-    a.bar = reinterpret_cast<uint32_t *>(tab + B.bar_at());
+    a.wins = reinterpret_cast<const NetWin *>(tab + B.wins_at(n));
+    a.tile_pre = reinterpret_cast<const uint32_t *>(tab + B.pre_at(n));
+    a.bar = reinterpret_cast<uint32_t *>(tab + B.bar_at(n));
     a.n_nets = (uint32_t)n;
     a.n_tiles = n_tiles;
     a.steps = (uint32_t)std::min<uint64_t>(window, most);
@@ -1216,7 +1217,7 @@ static int run_lockstep(snn_net *const *hs, const uint64_t *steps, int32_t n, co
     a.status = &reinterpret_cast<const NetDev *>(B.pinned[b])[first].rec->status;
     CU_TRY(launch_run(a, shape, L2Window{}, s));
     ++hs[0]->launches;
-    hs[0]->h2d += B.bytes();
+    hs[0]->h2d += B.bytes(n);
     for (int i = 0; i < n; ++i) {
       t_issue[i] += p.adv[i];
       left[i] -= p.adv[i];

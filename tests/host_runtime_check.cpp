@@ -220,8 +220,30 @@ static void check_footprint() {
     }
 }
 
+// What a set costs does not depend on the sets before it: its windows' tables
+// hold its own networks only.
+static void check_tables() {
+  const auto copied = [](std::vector<snn_handle> &hs) {
+    std::vector<uint64_t> steps(hs.size(), 30);
+    uint64_t bytes[2];
+    for (uint64_t &b : bytes) {
+      snn_stats st;
+      CHECK(snn_get_stats(hs[0], &st) == SNN_OK);
+      b = st.h2d_bytes;
+      if (&b == bytes) CHECK(snn_run_batch(hs.data(), steps.data(), (int)hs.size()) == SNN_OK);
+    }
+    return bytes[1] - bytes[0];
+  };
+  auto two = networks(2, 20, 1, 10), many = networks(100, 20, 1, 10);
+  const uint64_t before = copied(two);
+  CHECK(copied(many) > 20 * before);
+  CHECK(copied(two) == before);
+  free_all(two);
+  free_all(many);
+}
+
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}, {"large", check_large}, {"footprint", check_footprint}};
+  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}, {"large", check_large}, {"footprint", check_footprint}, {"tables", check_tables}};
   if (argc != 2 || !checks.count(argv[1])) return 2;
   checks.at(argv[1])();
   std::puts("ok");
