@@ -182,8 +182,9 @@ int snn_run_batch(const snn_handle *hs, const uint64_t *steps, int32_t n);
 
 /* Advance n networks by steps[i] each on launch path 0 (for all of them, else
  * SNN_ERR_ARG).  Networks that all have the default shape advance as in
- * snn_run_batch, except two large ones (500k neurons or more each, smallest
- * delay 1) on different streams in a call of two windows or more.  In that
+ * snn_run_batch, except two large ones (500k neurons or more each, below 700k
+ * none of more than 1.5 times the other; smallest delay 1) on different streams
+ * in a call of two windows or more.  In that
  * case, and with any other shape, every network runs on its own stream: the
  * windows of the networks are issued round robin, so kernels of different
  * networks run at the same time when their streams differ (networks sharing a

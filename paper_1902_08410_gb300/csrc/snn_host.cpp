@@ -1329,19 +1329,28 @@ static int run_set(snn_net *const *hs, const uint64_t *steps, int32_t n) {
 // Two large networks that leave the form to the library run as two kernels per
 // step on their own streams: one network's deliveries fill the time in which
 // the other waits, where in one launch both wait for the most active block.
-// One launch and apart, us a step, SWA + AW (AW + AW in brackets): two of 320k
-// neurons 12.2 and 12.2 (11.6 and 12.1), 500k 16.6 and 15.6 (15.8 and 15.7),
-// 720k 23.9 and 21.5 (22.6 and 20.0), 1.28M 39.0 and 34.4, 2M 57.2 and 55.1
-// (46.1 and 46.5); 1.28M beside 720k 31.4 and 32.3; four of 320k 21.6 and 27.7.
-// In the windows' graphs the steps past the end of a call cost launches, so the
-// call has at least two windows.
+// One launch and apart, us a step, SWA + AW (AW + AW in brackets), networks of
+// 320k (16x16 modules), 500k (20x20) .. neurons:
+//   320k + 320k    11.1 and 11.7 (10.2 and 11.1)    500k + 320k    13.3 and 13.4 (12.8 and 13.7)
+//   500k + 500k    14.9 and 14.6 (14.4 and 15.0)    720k + 500k    18.0 and 17.2 (17.1 and 16.8)
+//   605k + 605k    17.3 and 16.8 (17.3 and 17.1)    980k + 500k    21.5 and 21.9 (20.7 and 21.7)
+//   720k + 720k    20.5 and 19.0 (20.1 and 19.4)    980k + 720k    25.8 and 22.8 (24.1 and 22.5)
+//   1.28M + 1.28M  36.7 and 32.4 (34.8 and 32.5)    1.28M + 720k   31.7 and 27.5 (30.0 and 25.8)
+//   2M + 2M        53.2 and 49.1 (50.1 and 50.0)    1.62M + 720k   40.8 and 32.7 (37.6 and 30.6)
+// Apart gains from about 600k neurons each, and with 500k beside a network of
+// similar size (at 500k + 500k it depends on the regimes); a network of 500k ends
+// its steps too early to fill the waits of one twice as large.  In the windows'
+// graphs the steps past the end of a call cost launches, so the call has at least
+// two windows.
 constexpr uint32_t kApartNeurons = 500000;
+constexpr uint32_t kApartAnySize = 700000;   // from here on beside one of any size, below of at most 1.5 times its own
 
 static bool run_apart(snn_net *const *hs, const uint64_t *steps, int32_t n) {
   if (n != 2 || hs[0]->stream == hs[1]->stream) return false;   // on one stream they would take turns
   for (int i = 0; i < n; ++i)
-    if (hs[i]->L.N < kApartNeurons || hs[i]->L.kmin != 1u || steps[i] < 2u * (uint64_t)plain_window(hs[i])) return false;
-  return true;
+    if (hs[i]->L.kmin != 1u || steps[i] < 2u * (uint64_t)plain_window(hs[i])) return false;
+  const uint64_t less = std::min(hs[0]->L.N, hs[1]->L.N), more = std::max(hs[0]->L.N, hs[1]->L.N);
+  return less >= kApartNeurons && (less >= kApartAnySize || 2u * more <= 3u * less);
 }
 
 // Networks of snn_run_concurrent: those that leave the form to the library

@@ -242,8 +242,25 @@ static void check_tables() {
   free_all(many);
 }
 
+// Which pairs run as two kernels per step on their own streams.
+static void check_pairs() {
+  const struct {
+    int a, b;
+    bool apart;
+  } pairs[] = {{400, 399, false}, {400, 400, true}, {400, 600, true}, {400, 601, false}, {559, 839, false}, {560, 841, true}};
+  for (const auto &p : pairs) {
+    std::vector<snn_handle> hs = {networks(1, 20, 1, 10, p.a)[0], networks(1, 20, 1, 10, p.b)[0]};
+    for (int i = 0; i < 2; ++i) hs[i]->stream = reinterpret_cast<cudaStream_t>(uintptr_t(i + 1));
+    const uint64_t steps[2] = {20, 20};
+    g_graph_streams.clear();
+    CHECK(snn_run_concurrent(hs.data(), steps, 2) == SNN_OK);
+    CHECK(!g_graph_streams.empty() == p.apart);
+    free_all(hs);
+  }
+}
+
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}, {"large", check_large}, {"footprint", check_footprint}, {"tables", check_tables}};
+  const std::map<std::string, void (*)()> checks = {{"phase", check_phase}, {"failure", check_failure}, {"large", check_large}, {"footprint", check_footprint}, {"tables", check_tables}, {"pairs", check_pairs}};
   if (argc != 2 || !checks.count(argv[1])) return 2;
   checks.at(argv[1])();
   std::puts("ok");

@@ -23,7 +23,7 @@ def exe(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("check", ["phase", "failure", "large", "footprint", "tables"])
+@pytest.mark.parametrize("check", ["phase", "failure", "large", "footprint", "tables", "pairs"])
 def test_host_runtime(exe, check):
     r = subprocess.run([exe, check], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
