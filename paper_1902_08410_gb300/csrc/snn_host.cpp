@@ -250,7 +250,6 @@ void build_inputs(const snn_params &p, BuildDev &bd) {
     }
   bd.n_delay = (uint32_t)p.n_delay;
   bd.min_delay = (uint32_t)(p.min_delay < 1 ? 1 : p.min_delay);
-  bd.p_local_mode = p.p_local >= 0.0f ? 1 : 0;
 }
 
 }  // namespace snn
@@ -283,7 +282,7 @@ int snn_validate_params(const snn_params &p) {
   if (!(p.lambda > 0.0f) || !std::isfinite(p.lambda)) return fail(SNN_ERR_ARG, "lambda must be > 0");
   if (!std::isfinite(p.p_local) || p.p_local > 1.0f) return fail(SNN_ERR_ARG, "p_local must be <= 1");
   if (p.out_degree < 1) return fail(SNN_ERR_ARG, "out_degree must be >= 1");
-  if (p.out_degree > 2048) return fail(SNN_ERR_LIMIT, "out_degree above 2048");
+  if (p.out_degree > kMaxM) return fail(SNN_ERR_LIMIT, "out_degree above " + std::to_string(kMaxM));
   if (p.n_delay < 1 || p.n_delay > 254) return fail(SNN_ERR_ARG, "n_delay must be in 1..254");
   if (p.min_delay < 0 || p.min_delay > p.n_delay) return fail(SNN_ERR_ARG, "min_delay must be in 0..n_delay");
   if (!(p.dt_ms > 0.0f)) return fail(SNN_ERR_ARG, "dt_ms must be > 0");
@@ -323,7 +322,7 @@ static Layout make_layout(const snn_params &p) {
   // so that this bound fits the entry budget, and the raster can never overflow.
   const size_t budget = std::min<size_t>(192ull << 20, std::max<size_t>(8ull << 20, (size_t)L.N * 256u));
   const size_t per_step = (size_t)L.N * 8u / (size_t)(narp_min + 1) + 8u;
-  L.window = (uint32_t)std::max<size_t>(16, std::min<size_t>(1024, budget / per_step));
+  L.window = (uint32_t)std::max<size_t>(16, std::min<size_t>(kMaxWindow, budget / per_step));
   L.rec_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFF0ull,
                                            (uint64_t)L.N * ((L.window + narp_min) / (narp_min + 1) + 1));
   L.rates_bins = L.window / (uint32_t)p.bin_steps + 2u;

@@ -12,7 +12,8 @@ constexpr int kK = 1250;          // neurons per module (Sec. 2.2)
 constexpr int kNPop = 3;          // F, B, I
 constexpr int kZTab = 4096;       // Gaussian quantile table size (12-bit index)
 constexpr int kPoisMax = 16;      // external events per neuron and step are capped at 16
-constexpr int kMaxM = 4096;       // out-degree limit
+constexpr int kMaxM = 2048;       // out-degree limit
+constexpr uint32_t kMaxWindow = 1024;   // steps of a window at most
 constexpr int kNeuronAlign = 128; // neuron arrays padded to a multiple of 128
 
 // status bits written by kernels
@@ -111,7 +112,6 @@ struct BuildDev {
   float sig[kNPop][kNPop];
   uint32_t n_delay;     // delays uniform on min_delay..n_delay
   uint32_t min_delay;
-  int32_t p_local_mode; // 1 when p_local >= 0 (local bucket shortcut valid), 0 otherwise
 };
 
 // ---- launchers (snn_kernels.cu) -------------------------------------------

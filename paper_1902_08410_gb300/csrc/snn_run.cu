@@ -47,6 +47,8 @@ constexpr uint32_t kPendCap = 1024;      // neurons with two or more external ev
 constexpr uint32_t kSpinLimit = 1u << 22;   // barrier polls (about a microsecond each) before giving up
 
 // Live spike: id (24 bits) | step of the window + 512 (12) | position in the row (12) | network (16).
+// A spike of a window before is at most 254 steps old at the window's start.
+static_assert(kMaxM < (1 << 12) && kMaxWindow + 512u <= (1u << 12), "fields of a live spike");
 __device__ __forceinline__ unsigned long long live_pack(uint32_t id, int kts, uint32_t p, uint32_t net) {
   return (unsigned long long)(id | ((p & 0xFFu) << 24)) |
          ((unsigned long long)((p >> 8) | ((uint32_t)(kts + 512) << 4) | (net << 16)) << 32);
