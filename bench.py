@@ -228,6 +228,13 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
+def neuron_bytes(form: str) -> float:
+    """Bytes per neuron and step that a form has to move: two kernels per step
+    read and write V, c and the refractory counter, read the input and clear it;
+    the persistent kernel ("batch") keeps the state in shared memory over a window."""
+    return 8.0 if form == "batch" else 26.0
+
+
 def committed_traffic(kernel: str) -> float | None:
     """DRAM bytes per launch from the committed ncu capture, if the kernel source is unchanged."""
     try:
@@ -485,7 +492,7 @@ def run_gb300(args, dist: Dist):
         rec_bytes = 8 if n.params["record_format"] == W.REC_F32 else 6
         timed_spk_per_step = spikes[j] / float(args.steps * steps)
         per_net.append({"step_ms": t_step / ns, "update_ms": t_upd / ns, "deliver_ms": t_dl / ns,
-                        "update_bytes": 26.0 * n.N,
+                        "update_bytes": neuron_bytes("two kernels") * n.N,
                         "deliver_bytes": timed_spk_per_step * (n.M * rec_bytes + 8),
                         "timed_spikes_per_step": timed_spk_per_step, "sampled_spikes_per_step": spk / ns})
     upd_ms = sum(x["update_ms"] for x in per_net) / len(per_net)
@@ -507,20 +514,20 @@ def run_gb300(args, dist: Dist):
         # the timed region ran both networks in one launch of the persistent
         # kernel per window: its figures are the timed region's per step
         fu_ms = 1e3 * elapsed / (args.steps * steps)
-        fu_b = sum(x["update_bytes"] + x["deliver_bytes"] for x in per_net)
+        fu_b = sum(neuron_bytes(form) * n.N + x["deliver_bytes"] for n, x in zip(nets, per_net))
         kernels["k_run"] = {"ms_per_launch": fu_ms, "algorithmic_bytes": fu_b,
                               "achieved_gbs": fu_b / (fu_ms * 1e-3) / 1e9}
         share["k_run"] = 1.0
         dom = "k_run"
         method = ("k_run: one launch per window for both networks in the timed region; ms_per_launch = timed "
-                  "region / steps (CUDA events on the launching stream; one step of a launch), bytes = both networks' neuron state + "
+                  "region / steps (CUDA events on the launching stream; one step of a launch), bytes = 8 per neuron (input read and cleared) + "
                   "timed-region spikes per step x (M x record bytes + 8).  k_update / k_deliver: the two-kernel "
                   "path of each network alone, for reference (" + method + ")")
     ach = kernels[dom]["achieved_gbs"]
     # the whole step, the unit a user sees: algorithmic bytes of a step (neuron
     # state + every record delivered) over the step time, per network alone,
     # and over the timed region for the job (both networks concurrently)
-    job_bytes = sum(26.0 * n.N * args.steps * steps for n in nets) + sum(
+    job_bytes = sum(neuron_bytes(form) * n.N * args.steps * steps for n in nets) + sum(
         spikes[j] * (nets[j].M * (8 if nets[j].params["record_format"] == W.REC_F32 else 6) + 8)
         for j in range(len(nets)))
     step_frac = {names[j]: (x["update_bytes"] + x["deliver_bytes"]) / (x["step_ms"] * 1e-3) / 1e9 / peak
@@ -875,7 +882,7 @@ def measure_grid64(snn, torch, dist: Dist, regime: str, lam: float, fmt: int, ti
     sim_s = timed * W.DT_MS * 1e-3
     rec_bytes = 8 if fmt == W.REC_F32 else 6
     peak, _ = measured_peaks()
-    step_bytes = 26.0 * net.N + spikes / timed * (net.M * rec_bytes + 8)
+    step_bytes = neuron_bytes("two kernels") * net.N + spikes / timed * (net.M * rec_bytes + 8)
     out = {"format": "f32" if fmt == W.REC_F32 else "i16", "regime": regime, "lambda": lam,
            "events_per_s": spikes * EQUIV_PER_SPIKE / sec, "sim_seconds_per_wall_second": sim_s / sec,
            "us_per_step": 1e6 * sec / timed, "steps_timed": timed, "rate_hz": spikes / (net.N * sim_s),
