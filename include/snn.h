@@ -175,8 +175,13 @@ int snn_run(snn_handle h, uint64_t steps);
  * snn_run on it alone.  The networks must share one device; a launch is ordered
  * on the stream of its first network, behind the others' streams, and ends
  * before the call returns.
+ * Networks advanced from different host threads run side by side only while a
+ * window's launch leaves room on the SMs (up to 4 x 128 neurons per SM in a
+ * network), else their windows take turns: eight of 8x8 modules 32 us a step,
+ * 11 us here.
  * Errors as snn_run, plus SNN_ERR_ARG (a network twice or NULL) and
- * SNN_ERR_LIMIT (more than 65535 networks).  The paper has no counterpart:
+ * SNN_ERR_LIMIT (more than 65535 networks).  After SNN_ERR_CUDA the networks
+ * whose steps were under way answer SNN_ERR_STATE.  The paper has no counterpart:
  * batching independent networks is a systems pattern of this library. */
 int snn_run_batch(const snn_handle *hs, const uint64_t *steps, int32_t n);
 
@@ -242,9 +247,9 @@ int snn_set_launch(snn_handle h, const snn_launch *cfg);
  * at least 3% faster.  Synchronises the network's stream. */
 int snn_autotune(snn_handle h, uint32_t trial_steps);
 
-/* The same with the launch path fixed: path 0 tunes the two-kernel path only
- * (the shapes snn_run_concurrent can run), 1 path 1 only, -1 both
- * (= snn_autotune).  The paper has no counterpart of the tuners. */
+/* The same with the launch path fixed: path 0 times two-kernel shapes only
+ * (beside the current one and the default, which leaves the form to the
+ * library), 1 path 1 only, -1 both (= snn_autotune).  The paper has no counterpart of the tuners. */
 int snn_autotune_path(snn_handle h, uint32_t trial_steps, int32_t path);
 
 /* The same for a batch advanced by snn_run_batch: path 1 shapes (threads per
