@@ -15,19 +15,23 @@
 //     delivered at a time, into as many input buffers: a group is 56 records on
 //     average, and reading each by itself costs DRAM an activation per 200 bytes
 //     and the SM more instructions to get at the records than to deliver them;
-//   * the grid meets once per step, or once per exchange period.  Between
+//   * the grid meets once per step, or once per exchange period or part of one.  Between
 //     arriving and waiting a block records its spikes, draws the next external
 //     drive and visits its live spikes; only the update and the delay-1 records
 //     of its new spikes stand between two barriers.
 //
 // What bounds it: small networks, the grid barrier and two L2 or DRAM round trips
 // a step (4x4 modules: 5.3 us a step as two kernels, 2.5 us here); larger ones,
-// the visits' reductions, about 3e11 a second in L2, beside the issue of update
-// and drive (24x24 modules at 8.7 Hz: 17.8 us as two kernels in the default
-// shape, 11.3 us here; 64 networks of 2.3M neurons in all: 78 us as one kernel
-// per step, 53 us here).  Measured beside it: one delay group per visit, 13-15 us
-// at 24x24; whole modules per block with the records of the own module summed in
-// shared memory, 17 us (blocks whose modules are active hold up the grid).
+// the visits and draws between two barriers.  Cycles of a step at 24x24 modules
+// and 8.7 Hz (17.8 us as two kernels in the default shape, 10.1-11.3 us here):
+// update 3000, records of new spikes 2900, visits and draws 9900, waiting for the
+// block's other warps and the other blocks 3900; at 4x4 200, 1500, 1200 and 3600.
+// The reductions by themselves are not the bound: 0.8e11 a second at 24x24, 1e11
+// with two such networks, where L2 took 2e11 to 3.7e11 scattered ones.  (64
+// networks of 2.3M neurons in all: 78 us as one kernel per step, 53 us here.)
+// Measured beside it: one delay group per visit, 13-15 us at 24x24; whole modules
+// per block with the records of the own module summed in shared memory, 17 us
+// (blocks whose modules are active hold up the grid).
 //
 // A window starts from the spike lists in global memory (hist, cnt) and leaves
 // its own last n_delay steps there, so the other launch paths can go on from
@@ -44,7 +48,9 @@ namespace snn {
 
 constexpr int kRunThreads = 640;
 constexpr uint32_t kPendCap = 1024;      // neurons with two or more external events listed per step and block
-constexpr uint32_t kSpinLimit = 1u << 22;   // barrier polls (about a microsecond each) before giving up
+// Barrier polls (about a microsecond each) before giving up.  The time that other streams' kernels hold SMs does not
+// count: a cooperative launch starts when all its blocks can be resident (it waited 25 s behind a kernel on four SMs).
+constexpr uint32_t kSpinLimit = 1u << 22;
 
 // Live spike: id (24 bits) | step of the window + 512 (12) | position in the row (12) | network (16).
 // A spike of a window before is at most 254 steps old at the window's start.
@@ -651,7 +657,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(const __grid_constant__ 
     // ---- delivery before the barrier
     const uint32_t tail = min(s.tail[ring], head + cap);
     const bool more = k + L < a.steps;
-    // Reductions are bound by the L2, the draws by issue: half of the warps begin with each.
+    // Visits wait for records and reductions, the draws for issue slots: half of the warps begin with each.
     auto visit_and_draw = [&](bool visits, uint32_t upto) {
       for (uint32_t i = 0; i < 2u; ++i) {
         if ((i ^ warp) & 1u) {
@@ -816,7 +822,7 @@ cudaError_t prepare_run_kernels() {
 // registers, no spills; 1024: 4-10% more time a step from 4x4 to 40x40 modules,
 // 512: 8% more from 16x16 on) but fewer for a few tiles, where the block barriers
 // cost more than further warps give.  The form fits as long as the state and `kmin` drives per
-// neuron stay in shared memory (2.1M neurons at kmin = 1); what does not fit
+// neuron stay in shared memory (2.35M neurons at kmin = 1); what does not fit
 // takes two kernels per step (64x64 modules: 80 us a step, against 125 and 217 us
 // in two forms of this kernel with the state in global memory).
 // `part`: a set that has too many drives for its whole exchange period keeps
