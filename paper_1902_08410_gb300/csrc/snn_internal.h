@@ -151,7 +151,6 @@ struct RunArgs {
   uint32_t steps;             // steps of the window (the longest of the networks)
   uint32_t nd_max;            // largest delay of the networks
   uint32_t kmin;              // smallest delay, the same for all networks
-  uint32_t phase;             // t0 mod kmin, the same for all networks that advance (those that have stopped: any)
   uint32_t visit;             // steps between two visits of a live spike (1 in the period form)
   uint32_t fifo;              // live spikes of one ring that a block holds in shared memory (power of two)
   uint32_t nt;                // tiles of a block, at most
@@ -160,6 +159,9 @@ struct RunArgs {
   // {grid barrier count, last step (+1) that overflowed a live list, lists not taken over}, zero at launch
   uint32_t *bar;
   uint32_t *status;           // status word of a network that advances
+  // t0 mod kmin, the same for all networks that advance (those that have stopped: any).  Last: among the fields above it
+  // moved what every step reads, 4x4 modules 2.375 us a step instead of 2.361
+  uint32_t phase;
 };
 struct RunShape {
   int blocks = 0, threads = 0;
